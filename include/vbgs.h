@@ -72,16 +72,18 @@ typedef enum {
 
 /* Option flags.  By default points (per frame) and components (by
  * posterior mean, refreshed every fourth frame) are processed in Morton
- * order, and the passes skip the (point tile, component tile) pairs whose
- * responsibilities are all below e^-t by a certified bound (pass 1: a bound
+ * order, and the passes skip pairs whose responsibilities are all below e^-t
+ * by a certified bound; a point then loses at most K e^-t of its mass.  The
+ * tensor-core forms skip (point tile, component tile) pairs (pass 1: a bound
  * of the tile's logits over the points' box against a lower bound of their
- * lse; pass 2: the tile maxima pass 1 measured); a point then loses at most
- * K e^-t of its mass: t = ln K + 37 in the FP64 form (~1e-16) and ln K + 20
- * in the FP32 and tensor-core forms (~2e-9, below FP32 resolution).
+ * lse; pass 2: the tile maxima pass 1 measured) with t = ln K + 20 (~2e-9,
+ * below FP32 resolution).  The CUDA-core forms skip single (point, component)
+ * pairs in every E-step (also vbgs_elbo, vbgs_reassign and
+ * vbgs_estep_noalloc) with t = ln K + 37 (~1e-16).
  * Neither changes a result beyond the form's rounding.  The plain form sets
  * both flags. */
 #define VBGS_FLAG_NO_REORDER 1   /* process in the caller's order */
-#define VBGS_FLAG_NO_SKIP    2   /* evaluate every tile in pass 2 */
+#define VBGS_FLAG_NO_SKIP    2   /* evaluate every pair (CUDA-core forms), every tile in pass 2 */
 #define VBGS_FLAG_PROPOSAL   4   /* learned candidate proposal (see vbgs_proposal_report) */
 #define VBGS_FLAG_SPLIT      8   /* the split model of Fig. 3 (below) */
 
@@ -371,9 +373,9 @@ int vbgs_profile_enable(vbgs_ctx *ctx, int on);
 int vbgs_profile_read(vbgs_ctx *ctx, double *ms, int64_t *launches, int reset);
 /* No paper counterpart (measurement).  Work counters of the profiled calls
  * since the last reset: pairs scored by
- * pass 1 (every pair in the CUDA-core forms; in the tensor-core forms the
- * pairs of the component tiles its certified bound did not rule out) and
- * pairs pass 2 evaluated (the ones its skip bound did not rule out).
+ * pass 1 (the pairs its certified bounds did not rule out: whole component
+ * tiles in the tensor-core forms; every pair with VBGS_FLAG_NO_SKIP in the
+ * CUDA-core forms) and pairs pass 2 evaluated (the same for its bounds).
  * Synchronises the stream. */
 int vbgs_profile_pairs(vbgs_ctx *ctx, int64_t *pass1_pairs, int64_t *pass2_pairs);
 const char *vbgs_profile_name(int i);

@@ -123,7 +123,7 @@ int ensure_capacity(vbgs_ctx *ctx, int64_t N)
         int64_t cap = std::max<int64_t>(N, 1024);
         if ((rc = dalloc(ctx, &ctx->d_X, (size_t)cap * VBGS_XS))) return rc;
         if ((rc = dalloc(ctx, &ctx->d_lse, (size_t)cap))) return rc;
-        if ((rc = dalloc(ctx, &ctx->d_lse_part, (size_t)(cap + 63) / 64 + 1))) return rc;
+        if ((rc = dalloc(ctx, &ctx->d_lse_part, (size_t)(cap + 31) / 32 + 1))) return rc;
         if ((rc = dalloc(ctx, &ctx->d_Xs, (size_t)cap * VBGS_XS))) return rc;
         if ((rc = dalloc(ctx, &ctx->d_pidx, (size_t)cap))) return rc;
         if ((rc = dalloc(ctx, &ctx->d_minlse, (size_t)(cap + 31) / 32 + 1))) return rc;
@@ -164,6 +164,13 @@ int ensure_capacity(vbgs_ctx *ctx, int64_t N)
             (rc = dalloc(ctx, &ctx->d_p1ub, tc_p1ub_floats(std::max<int64_t>(N, 1), ctx->K))))
             return rc;
         ctx->p1plan_cap = p1need;
+    }
+    if (!is_tc(ctx) && !(ctx->flags & VBGS_FLAG_NO_SKIP) && sparse_fits(N)) {
+        const size_t sneed = sparse_scratch_floats(N, ctx->K);
+        if (sneed > ctx->sparse_cap) {
+            if ((rc = dalloc(ctx, &ctx->d_sparse, sneed))) return rc;
+            ctx->sparse_cap = sneed;
+        }
     }
     size_t need = estep_cuda_core_scratch(std::max<int64_t>(N, 1), ctx->K, is_tc(ctx) ? VBGS_FP32 : ctx->precision);
     if (is_tc(ctx))   // pass-1 partials of up to 64 K-splits; pass-2 item partials
@@ -349,7 +356,9 @@ int order_frame(vbgs_ctx *ctx, int64_t N, bool points, bool comps = true)
 // Full E-step over N staged points X (N x 8) into lse (N) and ctx->d_dS.
 int run_estep_on(vbgs_ctx *ctx, const double *X, int64_t N, double *lse, bool want_stats, bool same_points = false)
 {
-    if (ctx->prof.on && !is_tc(ctx)) ctx->prof.pass1_pairs += N * (int64_t)ctx->K;   // tensor-core pass 1 counts on the device
+    // the tensor-core and sparse passes count on the device
+    if (ctx->prof.on && !is_tc(ctx) && ((ctx->flags & VBGS_FLAG_NO_SKIP) || !sparse_fits(N)))
+        ctx->prof.pass1_pairs += N * (int64_t)ctx->K;
     if (N == 0) {
         CU(cudaMemsetAsync(ctx->d_scal + SC_SUM_LSE, 0, sizeof(double), ctx->stream));
         if (want_stats) CU(cudaMemsetAsync(ctx->d_dS, 0, sizeof(double) * ctx->K * VBGS_F, ctx->stream));
@@ -369,6 +378,8 @@ int run_estep_on(vbgs_ctx *ctx, const double *X, int64_t N, double *lse, bool wa
     B.dS = ctx->d_dS;
     B.kperm = ctx->d_kperm;
     const bool skip = want_stats && !(ctx->flags & VBGS_FLAG_NO_SKIP);
+    if (!is_tc(ctx) && !(ctx->flags & VBGS_FLAG_NO_SKIP) && sparse_fits(N)) B.sparse = ctx->d_sparse;
+    B.same_points = same_points;
     B.tmax = skip ? ctx->d_tmax : nullptr;
     B.minlse = skip ? ctx->d_minlse : nullptr;
     B.skip_nats = (float)ctx->skip_nats;
@@ -890,7 +901,7 @@ void free_all(vbgs_ctx *ctx)
                     ctx->d_flags, ctx->d_X, ctx->d_lse, ctx->d_lse_part, ctx->d_part,
                     ctx->d_kperm, ctx->d_kinv, ctx->d_pidx, ctx->d_Xs, ctx->d_tmax, ctx->d_minlse,
                     ctx->sb.keys_in, ctx->sb.keys_out, ctx->sb.idx_in, ctx->sb.temp, ctx->d_tc_tiles, ctx->d_tc_hdr, ctx->d_plan,
-                    ctx->d_p1plan, ctx->d_p1ub, ctx->d_tile_dirty, ctx->d_Xhl, ctx->d_lse2f,
+                    ctx->d_p1plan, ctx->d_p1ub, ctx->d_tile_dirty, ctx->d_Xhl, ctx->d_lse2f, ctx->d_sparse,
                     ctx->d_pcache_next, ctx->d_rec_alt, ctx->d_rec32_alt, ctx->d_kinv_alt,
                     ctx->ra.k_in, ctx->ra.k_out, ctx->ra.i_in, ctx->ra.i_out, ctx->ra.pts, ctx->ra.comps,
                     ctx->ra.picks, ctx->ra.g, ctx->ra.v, ctx->ra.rows, ctx->ra.temp};

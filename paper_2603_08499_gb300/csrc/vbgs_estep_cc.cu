@@ -20,6 +20,7 @@
 // FP32 form: records in float and log2 units, ex2.approx on the MUFU, FP32
 // accumulation inside a split, FP64 partials and reduction.
 #include "vbgs_internal.cuh"
+#include "vbgs_pair.cuh"
 #include <algorithm>
 #include <mutex>
 #include <string>
@@ -31,44 +32,6 @@ namespace {
 constexpr int kThreads = 128;
 constexpr int kChunkK = 64;   // component records per shared-memory chunk (pass 1)
 constexpr int kChunkN = 64;   // points per shared-memory chunk (pass 2)
-
-__device__ __forceinline__ float ex2_approx(float x)
-{
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-template <typename T> struct Arith;
-template <> struct Arith<double> {
-    // r = exp(l - ref) in natural units
-    static __device__ __forceinline__ double expd(double v) { return exp(v); }
-    static __device__ __forceinline__ double lse_scale() { return 1.0; }
-};
-template <> struct Arith<float> {
-    // records are in log2 units: r = 2^(l2 - ref2)
-    static __device__ __forceinline__ float expd(float v) { return ex2_approx(v); }
-    static __device__ __forceinline__ float lse_scale() { return 1.4426950408889634f; }
-};
-
-// logit (without the -psi(sum alpha) term) of point x under record r:
-// c - 1/2 |M (x - m)|^2, M packed lower triangle at r[6..26].
-template <typename T>
-__device__ __forceinline__ T logit(const T *__restrict__ r, const T x[6])
-{
-    T d[6];
-#pragma unroll
-    for (int i = 0; i < 6; i++) d[i] = x[i] - r[i];
-    T q = T(0);
-#pragma unroll
-    for (int i = 0; i < 6; i++) {
-        T y = T(0);
-#pragma unroll
-        for (int j = 0; j <= i; j++) y = fma(r[6 + tri(i, j)], d[j], y);
-        q = fma(y, y, q);
-    }
-    return fma(T(-0.5), q, r[27]);
-}
 
 // Pass 1.  grid = (point blocks, K splits).  part[split * N + n] = (max, sum)
 // with max in natural units and sum = sum_k exp(l_k - max).  When tmax is
@@ -378,6 +341,12 @@ double skip_nats_for(int precision, int K)
     return std::max(t, 20.0);
 }
 
+void launch_reduce_splits(const double *part, int nsplit, int K, const float *anchor, const int *kperm, double *dS,
+                          cudaStream_t st)
+{
+    k_reduce_splits<<<(K + 127) / 128, 128, 0, st>>>(part, nsplit, K, anchor, kperm, dS);
+}
+
 int launch_block_sum(const double *part, int n, double *sum_out, cudaStream_t st, Prof *pf)
 {
     pf->begin(VBGS_PROF_MERGE, st);
@@ -437,6 +406,9 @@ int launch_estep_cuda_core(const EstepBuffers &B, int precision, bool want_stats
     const bool f64 = precision == VBGS_FP64;
     Plan pl = f64 ? make_plan<kPPT64>(B.N, B.K, sms) : make_plan<kPPT32>(B.N, B.K, sms);
     if (pl.scratch > B.part_cap) return -2;
+    if (B.sparse)
+        return launch_estep_sparse(B, precision, want_stats, pl.kps, pl.p1_splits, pl.nps, pl.p2_splits, sms,
+                                   reinterpret_cast<unsigned int *>(B.scal + SC_MERGE_DONE), st, pf);
     int launches = 0;
     double2 *p1 = reinterpret_cast<double2 *>(B.part);
     dim3 g1(pl.p1_blocks, pl.p1_splits);
@@ -648,21 +620,47 @@ extern "C" int vbgs_estep_noalloc(vbgs_ctx *ctx, const double *points, int64_t N
     pl.nps = (N + s2max - 1) / s2max;
     pl.p2_splits = (int)((N + pl.nps - 1) / pl.nps);
 
-    double2 *p1 = reinterpret_cast<double2 *>(part);
-    dim3 g1(pl.p1_blocks, pl.p1_splits);
-    if (f64) k_pass1<double, kPPT64><<<g1, kThreads, 0, st>>>(X, N, ctx->d_rec, K, pl.kps, p1, nullptr);
-    else     k_pass1<float, kPPT32><<<g1, kThreads, 0, st>>>(X, N, ctx->d_rec32, K, pl.kps, p1, nullptr);
-    k_merge<<<mb, 256, 0, st>>>(p1, pl.p1_splits, N, nullptr, lse_out, nullptr, nullptr);
-    dim3 g2(pl.p2_tiles, pl.p2_splits);
-    if (f64) k_pass2<double><<<g2, kThreads, 0, st>>>(X, lse_out, N, pl.nps, ctx->d_rec, K, part, nullptr, nullptr, 1, 1, nullptr,
-                                                        0.f);
-    else     k_pass2<float><<<g2, kThreads, 0, st>>>(X, lse_out, N, pl.nps, ctx->d_rec32, K, part, nullptr, nullptr, 1, 1, nullptr,
-                                                       0.f);
-    k_reduce_splits<<<(K + 127) / 128, 128, 0, st>>>(part, pl.p2_splits, K, f64 ? nullptr : ctx->d_rec32,
-                                                    ctx->d_kperm, dS_out);
+    // The sparse passes' scratch goes behind the partials of pass 1 (FP32
+    // form) and one slice of pass 2, where the array holds it; near the size
+    // limits the dense passes run.
+    const size_t part_need = std::max(f64 ? (size_t)0 : (size_t)pl.p1_splits * (size_t)N * 2, (size_t)K * 28);
+    const size_t sp_need = (sparse_scratch_floats(N, K) + 1) / 2;
+    const bool sparse = !(ctx->flags & VBGS_FLAG_NO_SKIP) && sparse_fits(N) && part_need + 32 + sp_need <= avail;
+    if (sparse) {
+        EstepBuffers B{};
+        B.X = X;
+        B.N = N;
+        B.K = K;
+        B.rec = ctx->d_rec;
+        B.rec32 = ctx->d_rec32;
+        B.lse = lse_out;
+        B.lse_part = nullptr;
+        B.part = part;
+        const size_t o_sp = (avail - sp_need) & ~size_t(31);
+        B.part_cap = o_sp;
+        B.sparse = reinterpret_cast<float *>(part + o_sp);
+        B.dS = dS_out;
+        B.kperm = ctx->d_kperm;
+        const int l = launch_estep_sparse(B, f64 ? VBGS_FP64 : VBGS_FP32, true, pl.kps, pl.p1_splits, pl.nps,
+                                          pl.p2_splits, sms, nullptr, st, &off);
+        if (l < 0) return noalloc_fail(ctx, VBGS_ECUDA, "vbgs_estep_noalloc: launch failed");
+        ctx->launches = 4 + l;   // memset + 2 staging kernels, the passes, lse shift
+    } else {
+        double2 *p1 = reinterpret_cast<double2 *>(part);
+        dim3 g1(pl.p1_blocks, pl.p1_splits);
+        if (f64) k_pass1<double, kPPT64><<<g1, kThreads, 0, st>>>(X, N, ctx->d_rec, K, pl.kps, p1, nullptr);
+        else     k_pass1<float, kPPT32><<<g1, kThreads, 0, st>>>(X, N, ctx->d_rec32, K, pl.kps, p1, nullptr);
+        k_merge<<<mb, 256, 0, st>>>(p1, pl.p1_splits, N, nullptr, lse_out, nullptr, nullptr);
+        dim3 g2(pl.p2_tiles, pl.p2_splits);
+        if (f64) k_pass2<double><<<g2, kThreads, 0, st>>>(X, lse_out, N, pl.nps, ctx->d_rec, K, part, nullptr, nullptr, 1, 1,
+                                                            nullptr, 0.f);
+        else     k_pass2<float><<<g2, kThreads, 0, st>>>(X, lse_out, N, pl.nps, ctx->d_rec32, K, part, nullptr, nullptr, 1, 1,
+                                                           nullptr, 0.f);
+        k_reduce_splits<<<(K + 127) / 128, 128, 0, st>>>(part, pl.p2_splits, K, f64 ? nullptr : ctx->d_rec32,
+                                                        ctx->d_kperm, dS_out);
+        ctx->launches = 8;   // memset + 2 staging kernels, pass 1, merge, pass 2, reduce, lse shift
+    }
     k_lse_subtract_psi<<<mb, 256, 0, st>>>(lse_out, N, ctx->d_scal);
     if (cudaGetLastError() != cudaSuccess) return noalloc_fail(ctx, VBGS_ECUDA, "vbgs_estep_noalloc: launch failed");
-    // memset + 2 staging kernels, pass 1, merge, pass 2, reduce, lse shift
-    ctx->launches = 8;
     return VBGS_OK;
 }

@@ -214,6 +214,8 @@ struct EstepBuffers {
     float *tmax;          // pass-1 tile maxima [N/256][K/64] (nullptr: no skipping)
     float *minlse;        // per 256-point block min of lse
     float skip_nats;      // skip threshold t (skip_nats_for)
+    float *sparse = nullptr;   // CUDA-core forms: scratch of the sparse passes (nullptr: the dense ones)
+    bool same_points = false;  // X and N are the previous call's with this scratch
 };
 
 // ---- kernels / launchers (return number of launches, or -1 on error) ----
@@ -273,6 +275,16 @@ int launch_check_frame(const double *dS, int K, const double *X, int64_t N, cons
 int launch_estep_cuda_core(const EstepBuffers &B, int precision, bool want_stats, cudaStream_t st,
                            Prof *pf);
 size_t estep_cuda_core_scratch(int64_t N, int K, int precision);
+// The sparse passes (vbgs_estep_sparse.cu): the pairs above e^-(ln K + 37) of
+// a point's mass.  kps, p1_splits, nps, p2_splits: the dense passes' splits,
+// whose FP32 partial sums the FP32 form keeps.  done: finished-block counter
+// of the lse sum (zero between calls).  Without want_stats only lse.
+bool sparse_fits(int64_t N);
+size_t sparse_scratch_floats(int64_t N, int K);
+int launch_estep_sparse(const EstepBuffers &B, int precision, bool want_stats, int kps, int p1_splits, int64_t nps,
+                        int p2_splits, int num_sms, unsigned int *done, cudaStream_t st, Prof *pf);
+void launch_reduce_splits(const double *part, int nsplit, int K, const float *anchor, const int *kperm, double *dS,
+                          cudaStream_t st);
 int launch_lse_merge(const double2 *part, int nsplit, int64_t N, const int *item_start, double *lse,
                      double *lse_part, float *minlse, double *sum_out, cudaStream_t st, Prof *pf);
 int launch_pass2_fp32(const EstepBuffers &B, int tpb, int tkc, cudaStream_t st, Prof *pf);
@@ -514,6 +526,8 @@ struct vbgs_ctx {
     float *d_p1ub = nullptr;               // pass-1 logit bounds per (point tile, component tile)
     float *d_Xhl = nullptr;                // points as FP32 hi/lo pairs (tensor-core builders)
     float *d_lse2f = nullptr;              // lse in log2 units, FP32 (tensor-core pass 2)
+    float *d_sparse = nullptr;             // scratch of the sparse CUDA-core passes
+    size_t sparse_cap = 0;
     int64_t xhl_cap = 0;
     size_t p1plan_cap = 0;
     float *d_tc_hdr = nullptr;

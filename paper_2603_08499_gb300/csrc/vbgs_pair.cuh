@@ -1,0 +1,79 @@
+// vbgs_pair.cuh -- the logit of one (point, component) pair on the CUDA cores,
+// shared by the dense passes (vbgs_estep_cc.cu) and the sparse ones
+// (vbgs_estep_sparse.cu).
+#pragma once
+#include "vbgs_internal.cuh"
+
+namespace vbgs {
+
+__device__ __forceinline__ float ex2_approx(float x)
+{
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+template <typename T> struct Arith;
+template <> struct Arith<double> {
+    // r = exp(l - ref) in natural units
+    static __device__ __forceinline__ double expd(double v) { return exp(v); }
+    static __device__ __forceinline__ double lse_scale() { return 1.0; }
+};
+template <> struct Arith<float> {
+    // records are in log2 units: r = 2^(l2 - ref2)
+    static __device__ __forceinline__ float expd(float v) { return ex2_approx(v); }
+    static __device__ __forceinline__ float lse_scale() { return 1.4426950408889634f; }
+};
+
+// logit (without the -psi(sum alpha) term) of point x under record r:
+// c - 1/2 |M (x - m)|^2, M packed lower triangle at r[6..26].
+template <typename T>
+__device__ __forceinline__ T logit(const T *__restrict__ r, const T x[6])
+{
+    T d[6];
+#pragma unroll
+    for (int i = 0; i < 6; i++) d[i] = x[i] - r[i];
+    T q = T(0);
+#pragma unroll
+    for (int i = 0; i < 6; i++) {
+        T y = T(0);
+#pragma unroll
+        for (int j = 0; j <= i; j++) y = fma(r[6 + tri(i, j)], d[j], y);
+        q = fma(y, y, q);
+    }
+    return fma(T(-0.5), q, r[27]);
+}
+
+// The first three rows (position only) of the same quadratic form, and the
+// rest of it from there: the two halves together are logit's operations in
+// logit's order.
+__device__ __forceinline__ float quad_pos(const float *__restrict__ r, const float x[6])
+{
+    float d[3], q = 0.f;
+#pragma unroll
+    for (int i = 0; i < 3; i++) d[i] = x[i] - r[i];
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        float y = 0.f;
+#pragma unroll
+        for (int j = 0; j <= i; j++) y = fmaf(r[6 + tri(i, j)], d[j], y);
+        q = fmaf(y, y, q);
+    }
+    return q;
+}
+__device__ __forceinline__ float quad_rest(const float *__restrict__ r, const float x[6], float q)
+{
+    float d[6];
+#pragma unroll
+    for (int i = 0; i < 6; i++) d[i] = x[i] - r[i];
+#pragma unroll
+    for (int i = 3; i < 6; i++) {
+        float y = 0.f;
+#pragma unroll
+        for (int j = 0; j <= i; j++) y = fmaf(r[6 + tri(i, j)], d[j], y);
+        q = fmaf(y, y, q);
+    }
+    return q;
+}
+
+} // namespace vbgs
