@@ -165,8 +165,8 @@ int ensure_capacity(vbgs_ctx *ctx, int64_t N)
             return rc;
         ctx->p1plan_cap = p1need;
     }
-    if (!is_tc(ctx) && !(ctx->flags & VBGS_FLAG_NO_SKIP) && sparse_fits(N)) {
-        const size_t sneed = sparse_scratch_floats(N, ctx->K);
+    if (!is_tc(ctx) && !(ctx->flags & VBGS_FLAG_NO_SKIP) && sparse_fits(N, ctx->K)) {
+        const size_t sneed = sparse_scratch_floats(N, ctx->K, sparse_phi(N, ctx->precision));
         if (sneed > ctx->sparse_cap) {
             if ((rc = dalloc(ctx, &ctx->d_sparse, sneed))) return rc;
             ctx->sparse_cap = sneed;
@@ -357,7 +357,7 @@ int order_frame(vbgs_ctx *ctx, int64_t N, bool points, bool comps = true)
 int run_estep_on(vbgs_ctx *ctx, const double *X, int64_t N, double *lse, bool want_stats, bool same_points = false)
 {
     // the tensor-core and sparse passes count on the device
-    if (ctx->prof.on && !is_tc(ctx) && ((ctx->flags & VBGS_FLAG_NO_SKIP) || !sparse_fits(N)))
+    if (ctx->prof.on && !is_tc(ctx) && ((ctx->flags & VBGS_FLAG_NO_SKIP) || !sparse_fits(N, ctx->K)))
         ctx->prof.pass1_pairs += N * (int64_t)ctx->K;
     if (N == 0) {
         CU(cudaMemsetAsync(ctx->d_scal + SC_SUM_LSE, 0, sizeof(double), ctx->stream));
@@ -378,7 +378,8 @@ int run_estep_on(vbgs_ctx *ctx, const double *X, int64_t N, double *lse, bool wa
     B.dS = ctx->d_dS;
     B.kperm = ctx->d_kperm;
     const bool skip = want_stats && !(ctx->flags & VBGS_FLAG_NO_SKIP);
-    if (!is_tc(ctx) && !(ctx->flags & VBGS_FLAG_NO_SKIP) && sparse_fits(N)) B.sparse = ctx->d_sparse;
+    if (!is_tc(ctx) && !(ctx->flags & VBGS_FLAG_NO_SKIP) && sparse_fits(N, ctx->K)) B.sparse = ctx->d_sparse;
+    B.sparse_phi = sparse_phi(N, ctx->precision);
     B.same_points = same_points;
     B.tmax = skip ? ctx->d_tmax : nullptr;
     B.minlse = skip ? ctx->d_minlse : nullptr;
@@ -1016,7 +1017,7 @@ extern "C" int vbgs_update_batched(vbgs_ctx *const *scenes, int n_scenes, const 
             return fail(nullptr, VBGS_EINVAL, "vbgs_update_batched: scene %d uses the proposal (host-driven fallback)", i);
     }
     std::lock_guard<std::mutex> lock(g_batch.mu);
-    if (batch_streams(n_scenes) || tc_set_attributes())
+    if (batch_streams(n_scenes) || tc_set_attributes() || sparse_set_attributes())
         return fail(nullptr, VBGS_ECUDA, "vbgs_update_batched: stream set-up failed");
     vbgs_ctx *ctx = nullptr;   // for CU() error reporting
     // Every scene runs on a stream of the pool for the duration of the call,

@@ -341,12 +341,6 @@ double skip_nats_for(int precision, int K)
     return std::max(t, 20.0);
 }
 
-void launch_reduce_splits(const double *part, int nsplit, int K, const float *anchor, const int *kperm, double *dS,
-                          cudaStream_t st)
-{
-    k_reduce_splits<<<(K + 127) / 128, 128, 0, st>>>(part, nsplit, K, anchor, kperm, dS);
-}
-
 int launch_block_sum(const double *part, int n, double *sum_out, cudaStream_t st, Prof *pf)
 {
     pf->begin(VBGS_PROF_MERGE, st);
@@ -624,8 +618,10 @@ extern "C" int vbgs_estep_noalloc(vbgs_ctx *ctx, const double *points, int64_t N
     // form) and one slice of pass 2, where the array holds it; near the size
     // limits the dense passes run.
     const size_t part_need = std::max(f64 ? (size_t)0 : (size_t)pl.p1_splits * (size_t)N * 2, (size_t)K * 28);
-    const size_t sp_need = (sparse_scratch_floats(N, K) + 1) / 2;
-    const bool sparse = !(ctx->flags & VBGS_FLAG_NO_SKIP) && sparse_fits(N) && part_need + 32 + sp_need <= avail;
+    auto sp_size = [&](bool phi) { return (sparse_scratch_floats(N, K, phi) + 1) / 2; };
+    const bool phi = sparse_phi(N, ctx->precision) && part_need + 32 + sp_size(true) <= avail;
+    const size_t sp_need = sp_size(phi);
+    const bool sparse = !(ctx->flags & VBGS_FLAG_NO_SKIP) && sparse_fits(N, ctx->K) && part_need + 32 + sp_need <= avail;
     if (sparse) {
         EstepBuffers B{};
         B.X = X;
@@ -638,6 +634,7 @@ extern "C" int vbgs_estep_noalloc(vbgs_ctx *ctx, const double *points, int64_t N
         B.part = part;
         const size_t o_sp = (avail - sp_need) & ~size_t(31);
         B.part_cap = o_sp;
+        B.sparse_phi = phi;
         B.sparse = reinterpret_cast<float *>(part + o_sp);
         B.dS = dS_out;
         B.kperm = ctx->d_kperm;

@@ -55,6 +55,28 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
+// The same with thread-block clusters of `cluster` blocks.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, unsigned cluster, size_t smem,
+                                      cudaStream_t st, Args &&...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
 // Offsets into the packed lower triangle of a 6x6 matrix, row-major i >= j.
 __host__ __device__ constexpr int tri(int i, int j) { return i * (i + 1) / 2 + j; }
 // Offset of (i, j), i <= j, in the statistics upper triangle (after 1 + D).
@@ -215,6 +237,7 @@ struct EstepBuffers {
     float *minlse;        // per 256-point block min of lse
     float skip_nats;      // skip threshold t (skip_nats_for)
     float *sparse = nullptr;   // CUDA-core forms: scratch of the sparse passes (nullptr: the dense ones)
+    bool sparse_phi = false;   // the scratch has room for the feature table
     bool same_points = false;  // X and N are the previous call's with this scratch
 };
 
@@ -279,12 +302,12 @@ size_t estep_cuda_core_scratch(int64_t N, int K, int precision);
 // a point's mass.  kps, p1_splits, nps, p2_splits: the dense passes' splits,
 // whose FP32 partial sums the FP32 form keeps.  done: finished-block counter
 // of the lse sum (zero between calls).  Without want_stats only lse.
-bool sparse_fits(int64_t N);
-size_t sparse_scratch_floats(int64_t N, int K);
+bool sparse_fits(int64_t N, int K);
+int sparse_set_attributes();
+size_t sparse_scratch_floats(int64_t N, int K, bool phi);
+bool sparse_phi(int64_t N, int precision);   // whether a context keeps the FP64 form's feature table
 int launch_estep_sparse(const EstepBuffers &B, int precision, bool want_stats, int kps, int p1_splits, int64_t nps,
                         int p2_splits, int num_sms, unsigned int *done, cudaStream_t st, Prof *pf);
-void launch_reduce_splits(const double *part, int nsplit, int K, const float *anchor, const int *kperm, double *dS,
-                          cudaStream_t st);
 int launch_lse_merge(const double2 *part, int nsplit, int64_t N, const int *item_start, double *lse,
                      double *lse_part, float *minlse, double *sum_out, cudaStream_t st, Prof *pf);
 int launch_pass2_fp32(const EstepBuffers &B, int tpb, int tkc, cudaStream_t st, Prof *pf);
