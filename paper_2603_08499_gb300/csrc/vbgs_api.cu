@@ -126,6 +126,7 @@ int ensure_capacity(vbgs_ctx *ctx, int64_t N)
         if ((rc = dalloc(ctx, &ctx->d_lse_part, (size_t)(cap + 31) / 32 + 1))) return rc;
         if ((rc = dalloc(ctx, &ctx->d_Xs, (size_t)cap * VBGS_XS))) return rc;
         if ((rc = dalloc(ctx, &ctx->d_pidx, (size_t)cap))) return rc;
+        if ((rc = dalloc(ctx, &ctx->d_lse_s, (size_t)cap))) return rc;
         if ((rc = dalloc(ctx, &ctx->d_minlse, (size_t)(cap + 31) / 32 + 1))) return rc;
         ctx->ncap = cap;
     }
@@ -202,8 +203,8 @@ int ensure_reassign(vbgs_ctx *ctx, int64_t n)
     if ((rc = dalloc(ctx, &r.k_in, (size_t)cap)) || (rc = dalloc(ctx, &r.k_out, (size_t)cap)) ||
         (rc = dalloc(ctx, &r.i_in, (size_t)cap)) || (rc = dalloc(ctx, &r.i_out, (size_t)cap)) ||
         (rc = dalloc(ctx, &r.pts, (size_t)cap)) || (rc = dalloc(ctx, &r.comps, (size_t)cap)) ||
-        (rc = dalloc(ctx, &r.picks, (size_t)cap * 2)) || (rc = dalloc(ctx, &r.g, (size_t)cap)) ||
-        (rc = dalloc(ctx, &r.v, (size_t)cap)) || (rc = dalloc(ctx, &r.rows, (size_t)cap * 6)))
+        (rc = dalloc(ctx, &r.k_tie, (size_t)cap)) || (rc = dalloc(ctx, &r.g, (size_t)cap)) ||
+        (rc = dalloc(ctx, &r.v, (size_t)cap)) || (rc = dalloc(ctx, &r.rows, (size_t)cap * 7 + 1)))
         return rc;
     unsigned char *t = nullptr;
     const size_t tb = reassign_temp_bytes(cap);
@@ -275,6 +276,7 @@ int run_mstep(vbgs_ctx *ctx, const double *dS, bool write_next = false)
 {
     int rc;
     if ((rc = join_side(ctx))) return rc;
+    ctx->records_current = ctx->prior_cached = false;
     if (!dS) ctx->next_prior_ready = false;
     // the list the last E-step built belongs to these statistics only
     const bool listed = dS == ctx->d_dS && ctx->mstep_listed;
@@ -295,13 +297,43 @@ int run_mstep(vbgs_ctx *ctx, const double *dS, bool write_next = false)
     return VBGS_OK;
 }
 
+// The prior cache of the next frame, from the last M-step's slots.
+int apply_next(vbgs_ctx *ctx)
+{
+    const int l = launch_apply_next(ctx->K, ctx->d_pcache_next, ctx->d_pcache, ctx->stream, &ctx->prof);
+    if (l < 0) return fail(ctx, VBGS_ECUDA, "prior cache launch failed");
+    ctx->launches += l;
+    return VBGS_OK;
+}
+
+// The posterior prior0 (+) S_past for a call that only reads it.  After a
+// frame or an earlier such call the records and tiles already hold it (the
+// commit made S_past bitwise the statistics of the last M-step), and only the
+// KL total of that M-step is not this posterior's 0.
+int read_posterior(vbgs_ctx *ctx)
+{
+    int rc;
+    if (!ctx->records_current) return run_mstep(ctx, nullptr);
+    if ((rc = join_side(ctx))) return rc;
+    CU(cudaMemsetAsync(ctx->d_scal + SC_KL_TOTAL, 0, sizeof(double), ctx->stream));
+    return VBGS_OK;
+}
+
+// After read_posterior and the check of its flags: an M-step it ran is valid.
+void posterior_read(vbgs_ctx *ctx)
+{
+    if (!ctx->records_current) ctx->records_current = ctx->prior_cached = true;
+}
+
 // The posterior entering a frame when the previous frame's last M-step left
 // it ready (next_prior_ready): the commit made S_past bitwise the statistics
 // that M-step used, so its posterior is this frame's effective prior and the
 // records already hold it.  Move the records to the new component order
 // (kinv_old: the positions before it), take the prior cache, KL = 0; the
 // psi(sum alpha) of that M-step stays (equal up to the order of the sum).
-int frame_start_from_next(vbgs_ctx *ctx, bool moved, const int *kinv_old)
+// apply: the last call was that frame; else the prior cache is already this
+// frame's (prior_cached).
+int frame_start_from_next(vbgs_ctx *ctx, bool moved, const int *kinv_old, bool apply)
 {
     int l;
     if (moved) {
@@ -313,9 +345,7 @@ int frame_start_from_next(vbgs_ctx *ctx, bool moved, const int *kinv_old)
         std::swap(ctx->d_rec32, ctx->d_rec32_alt);
         if (is_tc(ctx)) CU(cudaMemsetAsync(ctx->d_tile_dirty, 0x01, sizeof(int) * ((ctx->K + 127) / 128), ctx->stream));
     }
-    l = launch_apply_next(ctx->K, ctx->d_pcache_next, ctx->d_pcache, ctx->stream, &ctx->prof);
-    if (l < 0) return fail(ctx, VBGS_ECUDA, "prior cache launch failed");
-    ctx->launches += l;
+    if (apply && (l = apply_next(ctx))) return l;
     CU(cudaMemsetAsync(ctx->d_scal + SC_KL_TOTAL, 0, sizeof(double), ctx->stream));
     if (is_tc(ctx)) {
         l = launch_coef_tiles(ctx->d_rec, ctx->d_rec32, ctx->K, ctx->precision == VBGS_BF16X3, ctx->d_tc_tiles,
@@ -326,6 +356,7 @@ int frame_start_from_next(vbgs_ctx *ctx, bool moved, const int *kinv_old)
     return VBGS_OK;
 }
 
+constexpr int64_t kSortScore = 2048;   // fewer points make at most 16 tiles: the sort costs more than it saves
 constexpr int kResortFrames = 4;   // frames between refreshes of the components' Morton order
 
 // Whether this frame refreshes the components' Morton order.
@@ -339,6 +370,7 @@ int order_frame(vbgs_ctx *ctx, int64_t N, bool points, bool comps = true)
     if (ctx->flags & VBGS_FLAG_NO_REORDER) return VBGS_OK;
     int l;
     if (comps) {
+        ctx->records_current = ctx->prior_cached = false;   // until they are written at the new positions
         l = launch_comp_order(ctx->d_m0, ctx->d_Spast, ctx->K, ctx->mp.beta0, ctx->box, ctx->sb, ctx->d_kperm,
                               ctx->d_kinv, ctx->stream, &ctx->prof);
         if (l < 0) return fail(ctx, VBGS_ECUDA, "component ordering failed");
@@ -392,7 +424,8 @@ int run_estep_on(vbgs_ctx *ctx, const double *X, int64_t N, double *lse, bool wa
                                 ctx->d_p1plan, ctx->d_p1ub, ctx->d_flags, ctx->num_sms, ctx->tune_p1,
                                 ctx->d_tile_dirty + (ctx->K + 127) / 128, ctx->plan_epoch, &item_start, &seed_part,
                                 ctx->stream, &ctx->prof, ctx->tc_knobs, ctx->skip_nats,
-                                reinterpret_cast<unsigned int *>(ctx->d_scal + SC_P1_DONE));
+                                reinterpret_cast<unsigned int *>(ctx->d_scal + SC_P1_DONE),
+                                !want_stats && !(ctx->flags & VBGS_FLAG_NO_SKIP));
         ctx->plan_epoch = ctx->coef_epoch;
         ctx->prof.p1_last.alloc_gen = ctx->alloc_gen;
         if (l < 0) return fail(ctx, VBGS_ECUDA, "tensor-core pass 1 launch failed: %s", cudaGetErrorString(cudaGetLastError()));
@@ -796,6 +829,24 @@ int prop_estep(vbgs_ctx *ctx, int64_t N, bool last_iter)
     return VBGS_OK;
 }
 
+// The E-step of a call that scores points under the current posterior: lse in
+// the caller's order.  In Morton order the boxes of neighbouring points are
+// small (36,000 points, K = 50,000: pass 1 on the tensor cores 329 us on the
+// caller's image rows, 75 us sorted, for 40 us of sorting and scattering).
+int score_points(vbgs_ctx *ctx, int64_t N)
+{
+    int rc;
+    const bool sort = !(ctx->flags & (VBGS_FLAG_NO_REORDER | VBGS_FLAG_NO_SKIP)) && N >= kSortScore;
+    if (sort && (rc = order_frame(ctx, N, true, false))) return rc;
+    ctx->last_sorted = false;
+    if ((rc = run_estep_on(ctx, sort ? ctx->d_Xs : ctx->d_X, N, sort ? ctx->d_lse_s : ctx->d_lse, false))) return rc;
+    if (!sort) return VBGS_OK;
+    if (launch_scatter(ctx->d_lse_s, ctx->d_pidx, N, ctx->d_lse, ctx->stream, &ctx->prof) < 0)
+        return fail(ctx, VBGS_ECUDA, "lse scatter launch failed");
+    ctx->launches += 1;
+    return VBGS_OK;
+}
+
 // same_points: the points are those of the previous E-step of this frame
 // (their FP32 split and tile boxes are current).
 int run_estep(vbgs_ctx *ctx, int64_t N, bool want_stats, bool last_iter = false, bool same_points = false)
@@ -841,7 +892,7 @@ int update_prepare(vbgs_ctx *ctx, const double *points, int64_t N, int n_iters, 
 int update_enqueue(vbgs_ctx *ctx, int64_t N, int n_iters, bool carry_prior)
 {
     int rc;
-    const bool from_next = carry_prior && ctx->next_prior_ready;
+    const bool apply = ctx->next_prior_ready, from_next = carry_prior && (apply || ctx->prior_cached);
     const bool reorder = !(ctx->flags & VBGS_FLAG_NO_REORDER);
     // The components' Morton order is refreshed on every kResortFrames-th
     // frame of the context (their means move little from frame to frame, so
@@ -853,11 +904,12 @@ int update_enqueue(vbgs_ctx *ctx, int64_t N, int n_iters, bool carry_prior)
     ctx->mstep_listed = false;
     ctx->next_prior_ready = false;
     ctx->next_written = false;
+    ctx->records_current = ctx->prior_cached = false;
     if (from_next && resort) std::swap(ctx->d_kinv, ctx->d_kinv_alt);   // keep the old inverse order
     if ((rc = order_frame(ctx, N, true, resort))) return rc;
     // Posterior entering the frame: the effective prior prior0 (+) S_past.
     if (from_next) {
-        if ((rc = frame_start_from_next(ctx, resort, ctx->d_kinv_alt))) return rc;
+        if ((rc = frame_start_from_next(ctx, resort, ctx->d_kinv_alt, apply))) return rc;
     } else if ((rc = run_mstep(ctx, nullptr))) return rc;
     const bool prop = ctx->prop.on && N > 0;
     if (prop) {
@@ -902,10 +954,10 @@ void free_all(vbgs_ctx *ctx)
                     ctx->d_flags, ctx->d_X, ctx->d_lse, ctx->d_lse_part, ctx->d_part,
                     ctx->d_kperm, ctx->d_kinv, ctx->d_pidx, ctx->d_Xs, ctx->d_tmax, ctx->d_minlse,
                     ctx->sb.keys_in, ctx->sb.keys_out, ctx->sb.idx_in, ctx->sb.temp, ctx->d_tc_tiles, ctx->d_tc_hdr, ctx->d_plan,
-                    ctx->d_p1plan, ctx->d_p1ub, ctx->d_tile_dirty, ctx->d_Xhl, ctx->d_lse2f, ctx->d_sparse,
+                    ctx->d_p1plan, ctx->d_p1ub, ctx->d_tile_dirty, ctx->d_Xhl, ctx->d_lse2f, ctx->d_sparse, ctx->d_lse_s,
                     ctx->d_pcache_next, ctx->d_rec_alt, ctx->d_rec32_alt, ctx->d_kinv_alt,
                     ctx->ra.k_in, ctx->ra.k_out, ctx->ra.i_in, ctx->ra.i_out, ctx->ra.pts, ctx->ra.comps,
-                    ctx->ra.picks, ctx->ra.g, ctx->ra.v, ctx->ra.rows, ctx->ra.temp};
+                    ctx->ra.k_tie, ctx->ra.g, ctx->ra.v, ctx->ra.rows, ctx->ra.temp};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     {
@@ -1031,6 +1083,8 @@ extern "C" int vbgs_update_batched(vbgs_ctx *const *scenes, int n_scenes, const 
         CU(cudaEventRecord(g_batch.ev_own[i], own[i]));
         CU(cudaStreamWaitEvent(g_batch.pool[i], g_batch.ev_own[i], 0));
         scenes[i]->stream = g_batch.pool[i];
+        // (a replayed graph advances S_past without update_enqueue)
+        scenes[i]->records_current = scenes[i]->prior_cached = scenes[i]->next_prior_ready = false;
         prof_on[i] = scenes[i]->prof.on;
         scenes[i]->prof.on = false;   // no event records inside the graph
     }
@@ -1681,6 +1735,7 @@ int vbgs_update(vbgs_ctx *ctx, const double *points, int64_t N, int n_iters, dou
                            ctx->stream));
     if ((rc = check_flags(ctx))) return rc;
     ctx->next_prior_ready = ctx->next_written;   // the commit ran: the carried prior is exact
+    ctx->records_current = ctx->next_written;
     return VBGS_OK;
 }
 
@@ -1692,11 +1747,11 @@ int vbgs_elbo(vbgs_ctx *ctx, const double *points, int64_t N, double *elbo_out, 
     ctx->launches = 0;
     int rc;
     if ((rc = ensure_capacity(ctx, N)) || (rc = ensure_elbo(ctx, 1))) return rc;
-    if ((rc = stage_points(ctx, points, N))) return rc;
+    // points are checked while the E-step runs (it changes no state)
     CU(cudaMemsetAsync(ctx->d_flags, 0, sizeof(int) * FL_COUNT, ctx->stream));
-    ctx->last_sorted = false;
-    if ((rc = run_mstep(ctx, nullptr))) return rc;
-    if ((rc = run_estep(ctx, N, false))) return rc;
+    if ((rc = stage_points(ctx, points, N, true))) return rc;
+    if ((rc = read_posterior(ctx))) return rc;
+    if ((rc = score_points(ctx, N))) return rc;
     if ((rc = join_side(ctx))) return rc;
     if (launch_elbo(ctx->d_scal, N, ctx->d_elbo, ctx->stream, &ctx->prof) < 0)
         return fail(ctx, VBGS_ECUDA, "ELBO launch failed");
@@ -1704,6 +1759,7 @@ int vbgs_elbo(vbgs_ctx *ctx, const double *points, int64_t N, double *elbo_out, 
     ctx->last_N = N;
     CU(cudaMemcpyAsync(elbo_out, ctx->d_elbo, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
     if ((rc = check_flags(ctx))) return rc;
+    posterior_read(ctx);
     if (lse_out && N > 0) return vbgs_get_lse(ctx, lse_out, N);
     return VBGS_OK;
 }
@@ -1718,28 +1774,23 @@ int vbgs_reassign(vbgs_ctx *ctx, const double *points, int64_t N, int n, double 
     if (!(tau > 0.0) || !std::isfinite(tau)) return fail(ctx, VBGS_EINVAL, "tau must be finite and > 0");
     if (n == 0) return VBGS_OK;
     if (!points || !gumbel) return fail(ctx, VBGS_EINVAL, "points and gumbel are required");
-    for (int64_t i = 0; i < N; i++)
-        if (!std::isfinite(gumbel[i])) return fail(ctx, VBGS_EINVAL, "non-finite gumbel value at %lld", (long long)i);
-    if (comp_key)
-        for (int k = 0; k < K; k++)
-            if (!std::isfinite(comp_key[k])) return fail(ctx, VBGS_EINVAL, "non-finite comp_key value at %d", k);
     ctx->launches = 0;
     int rc;
     // the per-point ELBO term under the current posterior, as vbgs_elbo
     if ((rc = ensure_capacity(ctx, N)) || (rc = ensure_elbo(ctx, 1)) ||
         (rc = ensure_reassign(ctx, std::max<int64_t>(N, K))))
         return rc;
-    if ((rc = stage_points(ctx, points, N))) return rc;
     CU(cudaMemsetAsync(ctx->d_flags, 0, sizeof(int) * FL_COUNT, ctx->stream));
-    ctx->last_sorted = false;
-    if ((rc = run_mstep(ctx, nullptr))) return rc;
-    if ((rc = run_estep(ctx, N, false))) return rc;
+    if ((rc = stage_points(ctx, points, N, true))) return rc;
+    if ((rc = read_posterior(ctx))) return rc;
+    if ((rc = score_points(ctx, N))) return rc;
     if ((rc = join_side(ctx))) return rc;
     if (launch_elbo(ctx->d_scal, N, ctx->d_elbo, ctx->stream, &ctx->prof) < 0)
         return fail(ctx, VBGS_ECUDA, "ELBO launch failed");
     ctx->launches += 1;
     ctx->last_N = N;
-    if ((rc = check_flags(ctx))) return rc;   // before the prior changes
+    // the caller's variates reach the device while the E-step runs; the device
+    // checks them, and the prior changes only if the whole call is good
     ReassignBuffers &rb = ctx->ra;
     CU(cudaMemcpyAsync(rb.g, gumbel, sizeof(double) * (size_t)N, cudaMemcpyHostToDevice, ctx->stream));
     if (comp_key) CU(cudaMemcpyAsync(rb.v, comp_key, sizeof(double) * (size_t)K, cudaMemcpyHostToDevice, ctx->stream));
@@ -1754,14 +1805,37 @@ int vbgs_reassign(vbgs_ctx *ctx, const double *points, int64_t N, int n, double 
     a.n = n;
     a.inv_tau = 1.0 / tau;
     a.have_v = comp_key != nullptr;
+    a.flags = ctx->d_flags;
+    // The new means change the posterior of the picked components alone: their
+    // records and prior cache are computed again, the others stay.
+    const bool carried = ctx->next_prior_ready, was_read = ctx->records_current;
+    ctx->records_current = ctx->prior_cached = ctx->next_prior_ready = false;
+    if (carried && was_read && (rc = apply_next(ctx))) return rc;
     const int l = launch_reassign(a, rb, ctx->stream);
     if (l < 0) return fail(ctx, VBGS_ECUDA, "reassign launch failed");
     ctx->launches += l;
-    std::vector<int> picks((size_t)n * 2);
-    std::vector<double> rows((size_t)n * 6);
-    CU(cudaMemcpyAsync(picks.data(), rb.picks, sizeof(int) * picks.size(), cudaMemcpyDeviceToHost, ctx->stream));
-    CU(cudaMemcpyAsync(rows.data(), rb.rows, sizeof(double) * rows.size(), cudaMemcpyDeviceToHost, ctx->stream));
-    CU(cudaStreamSynchronize(ctx->stream));
+    int *status = reinterpret_cast<int *>(rb.rows + (size_t)n * 6) + (size_t)n * 2;
+    int lm = launch_mstep_some(ctx->mp, ctx->d_m0, ctx->d_Spast, rb.comps, n, ctx->d_kinv, ctx->d_rec, ctx->d_rec32,
+                               ctx->d_pcache, status + 1, is_tc(ctx) ? ctx->d_tile_dirty : nullptr, ctx->stream,
+                               &ctx->prof);
+    if (lm < 0) return fail(ctx, VBGS_ECUDA, "posterior update launch failed");
+    ctx->launches += lm;
+    if (is_tc(ctx)) {
+        lm = launch_coef_tiles(ctx->d_rec, ctx->d_rec32, K, ctx->precision == VBGS_BF16X3, ctx->d_tc_tiles,
+                               ctx->d_tc_hdr, ctx->d_tile_dirty, ++ctx->coef_epoch, ctx->stream, &ctx->prof);
+        if (lm < 0) return fail(ctx, VBGS_ECUDA, "coefficient tile launch failed");
+        ctx->launches += lm;
+    }
+    std::vector<double> got((size_t)n * 7 + 1);
+    CU(cudaMemcpyAsync(got.data(), rb.rows, sizeof(double) * got.size(), cudaMemcpyDeviceToHost, ctx->stream));
+    if ((rc = check_flags(ctx))) return rc;   // (the prior is unchanged)
+    const double *rows = got.data();
+    const int *picks = reinterpret_cast<const int *>(rows + (size_t)n * 6);
+    const int bad = picks[(size_t)n * 2], nonpd = picks[(size_t)n * 2 + 1];
+    // a posterior that is not positive definite under the new mean is the next
+    // frame's to report
+    if (!nonpd) ctx->records_current = ctx->prior_cached = true;
+    if (bad) return fail(ctx, VBGS_EINVAL, "non-finite %s value", bad & 1 ? "gumbel" : "comp_key");
     // the host copy of the prior means follows the device's
     for (int i = 0; i < n; i++)
         for (int d = 0; d < 6; d++) ctx->m0_h[(size_t)picks[(size_t)n + i] * 6 + d] = rows[(size_t)i * 6 + d];
@@ -1769,7 +1843,6 @@ int vbgs_reassign(vbgs_ctx *ctx, const double *points, int64_t N, int n, double 
         for (int i = 0; i < n; i++) picked_points[i] = picks[i];
     if (picked_comps)
         for (int i = 0; i < n; i++) picked_comps[i] = picks[(size_t)n + i];
-    ctx->next_prior_ready = false;   // the next frame starts from the new prior
     return VBGS_OK;
 }
 
@@ -1821,12 +1894,14 @@ int vbgs_set_stats(vbgs_ctx *ctx, const double *S)
     if (!S) return fail(ctx, VBGS_EINVAL, "S is NULL");
     for (size_t i = 0; i < (size_t)ctx->K * VBGS_F; i++)
         if (!std::isfinite(S[i])) return fail(ctx, VBGS_EINVAL, "non-finite statistic at %zu", i);
+    ctx->records_current = ctx->prior_cached = ctx->next_prior_ready = false;
     CU(cudaMemcpyAsync(ctx->d_Spast, S, sizeof(double) * ctx->K * VBGS_F, cudaMemcpyHostToDevice,
                        ctx->stream));
     CU(cudaMemsetAsync(ctx->d_flags, 0, sizeof(int) * FL_COUNT, ctx->stream));
     int rc = run_mstep(ctx, nullptr);
-    if (rc) return rc;
-    return check_flags(ctx);
+    if (rc || (rc = check_flags(ctx))) return rc;
+    posterior_read(ctx);
+    return VBGS_OK;
 }
 
 int vbgs_get_posterior(vbgs_ctx *ctx, double *alpha, double *beta, double *m, double *Winv, double *nu)
@@ -1927,7 +2002,8 @@ int vbgs_save_state(vbgs_ctx *ctx, const char *path)
     h.precision = ctx->precision;
     h.flags = ctx->flags;
     h.has_prop = ctx->prop.on ? 1 : 0;
-    h.next_prior_ready = ctx->next_prior_ready ? 1 : 0;
+    // bit 0: next_prior_ready, bit 1: records_current, bit 2: prior_cached
+    h.next_prior_ready = (ctx->next_prior_ready ? 1 : 0) | (ctx->records_current ? 2 : 0) | (ctx->prior_cached ? 4 : 0);
     h.coef_epoch = ctx->coef_epoch;
     h.plan_epoch = ctx->plan_epoch;
     h.tune_p1 = ctx->tune_p1;
@@ -2060,7 +2136,9 @@ int vbgs_load_state(vbgs_ctx **out, const char *path, const vbgs_options *opt)
         return fail(nullptr, VBGS_ECUDA, "vbgs_load_state: copy to the device failed");
     }
     ctx->m0_h = m0;
-    ctx->next_prior_ready = h.next_prior_ready != 0;
+    ctx->next_prior_ready = (h.next_prior_ready & 1) != 0;
+    ctx->records_current = (h.next_prior_ready & 2) != 0;
+    ctx->prior_cached = (h.next_prior_ready & 4) != 0;
     ctx->coef_epoch = h.coef_epoch;
     ctx->plan_epoch = h.plan_epoch;
     ctx->tune_p1 = h.tune_p1;

@@ -454,8 +454,9 @@ __global__ void __launch_bounds__(128) k_coef_tiles(const double *__restrict__ r
 // of each 32-point row block and 128-component tile.
 // seed (nullable): the seed launch's partials; each row's running maximum
 // starts at its seed maximum, and a 64-column batch whose largest logit lies
-// more than `drop` (log2 units) below the running maximum in every row of the
-// warp is not exponentiated.  With drop = log2 K + 25 the terms left out are
+// more than `drop` (log2 units; 0: none is left out) below the running maximum
+// in every row of the warp is not exponentiated.  With drop = log2 K + 25 the
+// terms left out are
 // at most K 2^-drop = 2^-25 of a row's sum over all components (the sum is at
 // least its largest term, 1 in units of the final maximum): below FP32
 // rounding of the sum.  Its tile maxima are still taken.  pairs (nullable):
@@ -488,6 +489,11 @@ __global__ void __launch_bounds__(kThreadsTC, 3) k_pass1_tc(const float *__restr
     const int P = item_tile[item];
     const int lo = item_lo[item];
     const int nt = item_hi[item] - lo;
+    if (nt == 0) {   // an empty split of the score lists
+        const int64_t n0 = (int64_t)P * kRows + tid;
+        if (tid < kRows && n0 < N) part[(size_t)item * kRows + tid] = make_float2(-INFINITY, 0.f);
+        return;
+    }
     auto tile_at = [&](int jj) -> int { return list ? list[(size_t)P * ntiles + lo + jj] : lo + jj; };
 
     if (tid == 0) {
@@ -609,7 +615,7 @@ __global__ void __launch_bounds__(kThreadsTC, 3) k_pass1_tc(const float *__restr
                 float cm = fmax3(fmax3(mx8[0], mx8[1], mx8[2]), fmax3(mx8[3], mx8[4], mx8[5]), fmaxf(mx8[6], mx8[7]));
                 cm *= scale;
                 tmx = fmaxf(tmx, cm);
-                if (seed && __all_sync(0xffffffffu, cm < mrun - drop)) continue;   // negligible in every row
+                if (drop > 0.f && __all_sync(0xffffffffu, cm < mrun - drop)) continue;   // negligible in every row
                 if (pairs) ecols += (unsigned long long)max(0, min(64, nvalid - c));
                 if (cm > mrun) {
                     srun *= ex2f(mrun - cm);
@@ -989,7 +995,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_p1_seed(int64_t N, int ntiles,
 {
     pdl_wait();
     const int P = blockIdx.x, t = threadIdx.x, lane = t & 31, w = t >> 5;
-    for (int i = t; i < 4 * ntiles; i += kPlanThreads) {
+    for (int i = t; tmax && i < 4 * ntiles; i += kPlanThreads) {
         const int64_t rb = (int64_t)P * 4 + i / ntiles;
         if (rb * 32 < N) tmax[rb * ntiles + i % ntiles] = -INFINITY;
     }
@@ -1018,6 +1024,76 @@ __global__ void __launch_bounds__(kPlanThreads) k_p1_seed(int64_t N, int ntiles,
         sitem_lo[P] = 0;
         sitem_hi[P] = 1;
         if (P == 0) *snitems = ptiles;
+    }
+}
+
+// The lists of an E-step without statistics (score: vbgs_elbo,
+// vbgs_reassign): the dense launch's work items, splits of C component tiles of
+// every point tile, with the tiles left out whose certified bound lies more
+// than the threshold below LB.  The threshold is the FP64 form's, ln K + 37:
+// the terms left out then do not change the FP32 rounding of a partial or of
+// the merge, and the lse is the dense launch's bit for bit.
+__global__ void __launch_bounds__(kPlanThreads) k_p1_plan_score(int64_t N, int ntiles, int ptiles, int C, int ns,
+                                                                const float2 *__restrict__ spart,
+                                                                const float *__restrict__ ub, int *__restrict__ list,
+                                                                float skip_log2, int *__restrict__ item_start,
+                                                                int *__restrict__ item_tile, int *__restrict__ item_lo,
+                                                                int *__restrict__ item_hi, int *__restrict__ nitems)
+{
+    pdl_wait();
+    const int P = blockIdx.x, t = threadIdx.x, lane = t & 31, w = t >> 5;
+    __shared__ float red[kPlanWarps];
+    __shared__ int wsum[kPlanWarps];
+    __shared__ int base_sh;
+    const float *u = ub + (size_t)P * ntiles;
+    int *row = list + (size_t)P * ntiles;
+    const int js = row[0];
+    float lb = INFINITY;   // as in k_p1_plan
+    if (t < kRows && (int64_t)P * kRows + t < N) {
+        const float2 q = spart[(size_t)P * kRows + t];
+        const float l = q.x + __log2f(q.y);
+        lb = l - (1.f + 1e-5f * fabsf(l));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) lb = fminf(lb, __shfl_xor_sync(0xffffffffu, lb, o));
+    if (lane == 0) red[w] = lb;
+    if (t == 0) base_sh = 0;
+    __syncthreads();
+    float LB = red[0];
+    for (int q = 1; q < kPlanWarps; q++) LB = fminf(LB, red[q]);
+    const float thr = LB - skip_log2;
+    for (int j0 = 0; j0 < ntiles; j0 += kPlanThreads) {
+        const int j = j0 + t;
+        // (a bound or threshold that is not a number keeps the tile)
+        const bool keep = j < ntiles && (j == js || !(u[j] < thr));
+        const unsigned bb = __ballot_sync(0xffffffffu, keep);
+        if (lane == 0) wsum[w] = __popc(bb);
+        __syncthreads();
+        int off = base_sh;
+        for (int i = 0; i < w; i++) off += wsum[i];
+        off += __popc(bb & ((1u << lane) - 1u));
+        if (keep) row[off] = j;
+        if (j < ntiles && j % C == 0) {   // the first tile of a split
+            const int it = P * ns + j / C;
+            item_tile[it] = P;
+            item_lo[it] = off;
+            if (j) item_hi[it - 1] = off;
+        }
+        __syncthreads();
+        if (t == 0) {
+            int tot = 0;
+            for (int i = 0; i < kPlanWarps; i++) tot += wsum[i];
+            base_sh += tot;
+        }
+        __syncthreads();
+    }
+    if (t == 0) {
+        item_hi[P * ns + ns - 1] = base_sh;
+        item_start[P] = P * ns;
+        if (P == ptiles - 1) {
+            item_start[ptiles] = ptiles * ns;
+            *nitems = ptiles * ns;
+        }
     }
 }
 
@@ -1881,7 +1957,7 @@ int launch_pass1_tc(const double *X, float *Xhl, bool same_points, int64_t N, in
                     size_t part_cap_doubles, float *tmax, int *p1plan, float *p1ub, int *flags, int num_sms,
                     int tiles_per_item, const int *tile_epoch, int since, const int **item_start_out,
                     const double **seed_part_out, cudaStream_t st, Prof *pf, uint32_t knobs, double skip_nats,
-                    unsigned int *plan_done)
+                    unsigned int *plan_done, bool score)
 {
     float2 *part = reinterpret_cast<float2 *>(part_buf);
     int launches = 0;
@@ -1927,8 +2003,12 @@ int launch_pass1_tc(const double *X, float *Xhl, bool same_points, int64_t N, in
     const float drop = (float)(std::log2((double)std::max(K, 2)) + 25.0);
     const float2 *seed_rows = nullptr;
     *seed_part_out = nullptr;
+    float score_drop = 0.f;
+    // the dense items' component tiles (build_items with every tile listed)
+    const int room = target > ptiles ? target - ptiles : 1;
+    const int C = (int)std::max<int64_t>(tmin, ((int64_t)ptiles * ntiles + room - 1) / room);
     pf->begin(VBGS_PROF_PLAN, st);
-    if (tmax) {
+    if (tmax || score) {
         float *boxes = p1ub + (size_t)ptiles * ntiles;
         if (!same_points) {   // the boxes of the previous E-step's points are current
             launch_pdl(k_p1_boxes, ptiles, kRows, 0, st, X, N, boxes);
@@ -1951,18 +2031,30 @@ int launch_pass1_tc(const double *X, float *Xhl, bool same_points, int64_t N, in
         seed_rows = spart;
         pf->end(st);
         pf->begin(VBGS_PROF_PLAN, st);
+        if (score) {
+            const double t = std::log((double)std::max(K, 1)) + 37.0;
+            launch_pdl(k_p1_plan_score, ptiles, kPlanThreads, 0, st, N, ntiles, ptiles, C, (ntiles + C - 1) / C,
+                       (const float2 *)spart, (const float *)p1ub, list, (float)(t * 1.4426950408889634), item_start,
+                       item_tile, item_lo, item_hi, nitems);
+            // a 64-column batch 31 log2 units below a row's running maximum adds
+            // less than 2^-25 to a sum of at least 1: no change in FP32
+            score_drop = std::max(drop, 32.f);
+            seed_rows = nullptr;   // every row starts as in the dense launch
+        } else {
         // its last block builds the main launch's work items
         launch_pdl(k_p1_plan, ptiles, kPlanThreads, 0, st, N, ntiles, (const float2 *)spart, (const float *)p1ub,
                    list, counts, (float)(skip_nats * 1.4426950408889634),
                    ItemsArgs{tmin, target, item_start, item_tile, item_lo, item_hi, nitems, plan_done, nullptr});
         *seed_part_out = reinterpret_cast<const double *>(spart);
+        }
     } else {
         launch_pdl(k_p2_items, 1, 1024, 0, st, (const int *)nullptr, ptiles, ntiles, tmin, target, item_start,
                    item_tile, item_lo, item_hi, nitems, (int *)nullptr);
     }
     pf->end(st);
     pf->begin(VBGS_PROF_PASS1, st);
-    const int *lst = tmax ? list : nullptr;
+    const int *lst = tmax || score ? list : nullptr;
+    const float main_drop = score ? score_drop : tmax ? drop : 0.f;
     {
         Pass1Launch &L = pf->p1_last;
         L.valid = true;
@@ -1985,12 +2077,12 @@ int launch_pass1_tc(const double *X, float *Xhl, bool same_points, int64_t N, in
         L.flags = flags;
         L.knobs = knobs;
         L.seed = seed_rows;
-        L.drop = drop;
+        L.drop = main_drop;
     }
-    pass1(target, lst, item_tile, item_lo, item_hi, nitems, part, seed_rows, drop);
+    pass1(target, lst, item_tile, item_lo, item_hi, nitems, part, seed_rows, main_drop);
     pf->end(st);
     *item_start_out = item_start;
-    return cudaGetLastError() == cudaSuccess ? launches + (tmax ? 5 : 2) : -1;
+    return cudaGetLastError() == cudaSuccess ? launches + (tmax || score ? 5 : 2) : -1;
 }
 
 int launch_lse_merge_tc(const double *part_buf, const double *seed_part, int64_t N, const int *item_start, double *lse,

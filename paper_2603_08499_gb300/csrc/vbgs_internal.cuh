@@ -185,11 +185,14 @@ struct SortBuffers {
 
 // reassign (vbgs_reassign.cu): 64-bit sort keys and indices for up to cap
 // points or components, the caller's Gumbel variates (g) and component tie
-// keys (v), the sorted points and components, and the picks for the host
-// (rows: n x 6 point coordinates; picks: n points, then n components).
+// keys (v), the chosen points and components, and one block for the host
+// (rows: n x 6 point coordinates, then as ints n points, n components and the
+// flag of a non-finite variate or key and that of a posterior that is not
+// positive definite under its new mean).
 struct ReassignBuffers {
     unsigned long long *k_in = nullptr, *k_out = nullptr;
-    int *i_in = nullptr, *i_out = nullptr, *pts = nullptr, *comps = nullptr, *picks = nullptr;
+    unsigned long long *k_tie = nullptr;
+    int *i_in = nullptr, *i_out = nullptr, *pts = nullptr, *comps = nullptr;
     double *g = nullptr, *v = nullptr, *rows = nullptr;
     void *temp = nullptr;
     size_t temp_bytes = 0;
@@ -205,6 +208,7 @@ struct ReassignArgs {
     int K = 0, n = 0;
     double inv_tau = 1.0;
     bool have_v = false;
+    const int *flags = nullptr;    // the E-step's flags: the prior changes only if all are zero
 };
 size_t reassign_temp_bytes(int64_t n);
 // Returns the kernel launches issued, or -1.
@@ -285,6 +289,15 @@ int launch_point_order(const double *X, int64_t N, const BoxParams &box, SortBuf
                        int *pidx, cudaStream_t st, Prof *pf);
 int launch_comp_order(const double *m0, const double *Spast, int K, double beta0, const BoxParams &box,
                       SortBuffers &sb, int *kperm, int *kinv, cudaStream_t st, Prof *pf);
+// The posterior prior0 (+) S_past of the n components `comps` alone, at their
+// positions kinv: records, prior cache (its lnGamma terms, which do not depend
+// on m0, stay), tile_dirty.  *nonpd: set to a component + 1 whose W^-1 is not
+// positive definite.
+int launch_mstep_some(const MstepParams &P, const double *m0, const double *Spast, const int *comps, int n,
+                      const int *kinv, double *rec, float *rec32, double *cache, int *nonpd, int *tile_dirty,
+                      cudaStream_t st, Prof *pf);
+// out[idx[i]] = v[i]
+int launch_scatter(const double *v, const int *idx, int64_t N, double *out, cudaStream_t st, Prof *pf);
 int launch_commit(double *Spast, const double *dS, int K, const int *flags, cudaStream_t st, Prof *pf);
 int launch_elbo(double *scal, int64_t N, double *elbo_out, cudaStream_t st, Prof *pf);
 // Consistency checks of a frame's results (options.checks): sets
@@ -354,13 +367,14 @@ int tc_set_attributes();
 // and point-tile boxes are reused; tile_epoch / since: only the bounds of
 // tiles built after epoch `since` are recomputed).  item_start_out: the item
 // table the lse merge reads; seed_part_out: the seed launch's partials
-// (nullptr without skipping).
+// (nullptr without skipping).  score (without tmax): lists for an E-step
+// without statistics, whose lse is the dense launch's.
 int launch_pass1_tc(const double *X, float *Xhl, bool same_points, int64_t N, int K, bool bf16,
                     const unsigned char *tiles, const float *hdr, const float *rec32, double *part_buf,
                     size_t part_cap_doubles, float *tmax, int *p1plan, float *p1ub, int *flags, int num_sms,
                     int tiles_per_item, const int *tile_epoch, int since, const int **item_start_out,
                     const double **seed_part_out, cudaStream_t st, Prof *pf, uint32_t knobs, double skip_nats,
-                    unsigned int *plan_done);
+                    unsigned int *plan_done, bool score);
 // lse from pass 1's FP32 item partials and the seed launch's (nullable),
 // minlse per 32 points, sum of lse.
 int launch_lse_merge_tc(const double *part_buf, const double *seed_part, int64_t N, const int *item_start, double *lse,
@@ -531,6 +545,10 @@ struct vbgs_ctx {
     // records hold the same posterior (at the positions of d_kinv).
     bool next_prior_ready = false;
     bool next_written = false;                 // this frame's last M-step wrote d_pcache_next
+    // The records and coefficient tiles hold prior0 (+) S_past (checked
+    // positive definite): vbgs_elbo and vbgs_reassign need no M-step.
+    bool records_current = false;
+    bool prior_cached = false;     // and the prior cache: a frame may start from them (as from next_prior_ready)
     double *d_pcache_next = nullptr;           // K x 40: the next frame's effective-prior cache
     double *d_rec_alt = nullptr;               // record buffers for a new component order
     float *d_rec32_alt = nullptr;
@@ -579,6 +597,7 @@ struct vbgs_ctx {
     int elbo_cap = 0;
     int64_t ncap = 0;
     double *d_X = nullptr, *d_lse = nullptr, *d_lse_part = nullptr;
+    double *d_lse_s = nullptr;       // lse of sorted points (score_points)
     size_t part_cap = 0;
     double *d_part = nullptr;
     int64_t last_N = 0;

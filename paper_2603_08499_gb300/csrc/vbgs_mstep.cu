@@ -385,6 +385,28 @@ __global__ void __launch_bounds__(64) k_mstep(MstepParams P, const double *__res
     mstep_thread(P, m0, Spast, dS, pos, k, zero, rec, rec32, pc, kls, flags, tile_dirty, nullptr);
 }
 
+// The same for n components alone (reassign's new means), one warp a block:
+// the chain of one component is the launch, so it spreads over the SMs.
+__global__ void __launch_bounds__(32) k_mstep_some(MstepParams P, const double *__restrict__ m0,
+                                                    const double *__restrict__ Spast, const int *__restrict__ comps, int n,
+                                                    const int *__restrict__ kinv, double *__restrict__ rec,
+                                                    float *__restrict__ rec32, double *__restrict__ pc,
+                                                    int *__restrict__ flags, int *__restrict__ tile_dirty)
+{
+    pdl_wait();
+    const int i = blockIdx.x * 32 + threadIdx.x;
+    if (i >= n) return;
+    const int k = comps[i];
+    mstep_thread(P, m0, Spast, nullptr, kinv[k], k, false, rec, rec32, pc, pc, flags, tile_dirty, nullptr);
+}
+
+__global__ void k_scatter(const double *__restrict__ v, const int *__restrict__ idx, int64_t N, double *__restrict__ out)
+{
+    pdl_wait();
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < N) out[idx[i]] = v[i];
+}
+
 // ---------------------------------------------------------------------------
 // M-step of an iteration (dS given).  Few components change in an iteration
 // (a few thousand of 50,000 on the room stream), and an FP64 instruction
@@ -1077,6 +1099,25 @@ int launch_move_records(const int *kperm, const int *kinv_old, int K, const doub
     pf->begin(VBGS_PROF_MSTEP, st);
     launch_pdl(k_move_records, (unsigned)(((int64_t)K * 16 + 255) / 256), 256, 0, st, kperm, kinv_old, K, rec, rec32,
                rec_dst, rec32_dst);
+    pf->end(st);
+    return cudaGetLastError() == cudaSuccess ? 1 : -1;
+}
+
+int launch_mstep_some(const MstepParams &P, const double *m0, const double *Spast, const int *comps, int n,
+                      const int *kinv, double *rec, float *rec32, double *cache, int *nonpd, int *tile_dirty,
+                      cudaStream_t st, Prof *pf)
+{
+    pf->begin(VBGS_PROF_MSTEP, st);
+    launch_pdl(k_mstep_some, (n + 31) / 32, 32, 0, st, P, m0, Spast, comps, n, kinv, rec, rec32, cache,
+               nonpd - FL_NONPD, tile_dirty);
+    pf->end(st);
+    return cudaGetLastError() == cudaSuccess ? 1 : -1;
+}
+
+int launch_scatter(const double *v, const int *idx, int64_t N, double *out, cudaStream_t st, Prof *pf)
+{
+    pf->begin(VBGS_PROF_MISC, st);
+    launch_pdl(k_scatter, (unsigned)((N + 255) / 256), 256, 0, st, v, idx, N, out);
     pf->end(st);
     return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
