@@ -158,6 +158,13 @@ def _host_f64(a, shape=None) -> np.ndarray:
     return a
 
 
+def _out(shape, dtype=np.float64) -> np.ndarray:
+    """An array the library fills whole, or the call raises: not cleared first
+    (clearing the 11 MB of K = 50,000 statistics took 190 of 260 us; the copy
+    from the device takes 73)."""
+    return np.empty(shape, dtype=dtype)
+
+
 def _dp(a: np.ndarray):
     return a.ctypes.data_as(_DP)
 
@@ -241,7 +248,7 @@ def vbgs_update(ctx, points, n_iters: int) -> np.ndarray:
 def vbgs_elbo(ctx, points, want_lse: bool = False):
     ptr, N, keep = _points_ptr(points)
     out = np.zeros(1)
-    lse = np.zeros(max(N, 1)) if want_lse else None
+    lse = _out(max(N, 1)) if want_lse else None
     _check(lib().vbgs_elbo(ctx, ptr, N, _dp(out), _dp(lse) if want_lse else None), ctx)
     del keep
     return (float(out[0]), lse[:N]) if want_lse else float(out[0])
@@ -266,15 +273,14 @@ def vbgs_reassign(ctx, points, n: int, gumbel, tau: float = 1.0, comp_key=None):
 
 
 def vbgs_get_posterior(ctx, K: int) -> dict:
-    out = {"alpha": np.zeros(K), "beta": np.zeros(K), "m": np.zeros((K, D)),
-           "Winv": np.zeros((K, D, D)), "nu": np.zeros(K)}
+    out = {"alpha": _out(K), "beta": _out(K), "m": _out((K, D)), "Winv": _out((K, D, D)), "nu": _out(K)}
     _check(lib().vbgs_get_posterior(ctx, _dp(out["alpha"]), _dp(out["beta"]), _dp(out["m"]),
                                     _dp(out["Winv"]), _dp(out["nu"])), ctx)
     return out
 
 
 def vbgs_get_stats(ctx, K: int) -> np.ndarray:
-    S = np.zeros((K, F))
+    S = _out((K, F))
     _check(lib().vbgs_get_stats(ctx, _dp(S)), ctx)
     return S
 
@@ -285,13 +291,13 @@ def vbgs_set_stats(ctx, S) -> None:
 
 
 def vbgs_get_frame_stats(ctx, K: int) -> np.ndarray:
-    S = np.zeros((K, F))
+    S = _out((K, F))
     _check(lib().vbgs_get_frame_stats(ctx, _dp(S)), ctx)
     return S
 
 
 def vbgs_get_lse(ctx, N: int) -> np.ndarray:
-    lse = np.zeros(max(N, 1))
+    lse = _out(max(N, 1))
     _check(lib().vbgs_get_lse(ctx, _dp(lse), N), ctx)
     return lse[:N]
 
@@ -495,7 +501,7 @@ def vbgs_render(ctx, cam: dict, reference=None, want_image: bool = True):
     device ms)."""
     W, H = int(cam["width"]), int(cam["height"])
     c = camera_array(cam)
-    img = np.zeros((H, W, 3), dtype=np.float32) if want_image else None
+    img = _out((H, W, 3), np.float32) if want_image else None
     ref = None
     if reference is not None:
         ref = np.ascontiguousarray(reference, dtype=np.float32)
