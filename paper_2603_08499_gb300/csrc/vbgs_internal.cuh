@@ -461,6 +461,10 @@ struct RenderBuffers {
     unsigned long long *ekey = nullptr, *ekey_s = nullptr;   // (tile << 32 | depth rank) per covered tile
     int *eval = nullptr, *eval_s = nullptr;
     int2 *range = nullptr;                      // per tile: [first, last) of its sorted entries
+    int *list = nullptr, *count = nullptr;      // drawn components; their number and that of the visible ones
+    int4 *rect_s = nullptr;                     // rectangles front to back
+    cudaEvent_t ev[4] = {};
+    size_t cap_list = 0, cap_count = 0, cap_rect_s = 0;
     float *img = nullptr, *ref = nullptr;
     double *part = nullptr, *out = nullptr;
     void *temp = nullptr;

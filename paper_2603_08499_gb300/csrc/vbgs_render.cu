@@ -15,12 +15,24 @@
 // with alpha < 1/255 skipped, black background.
 //
 // GB300 layout of the work:
-//   k_splat_prep   a thread per component: posterior (FP64, from S_past and
-//                  the prior), camera transform, screen covariance and its
+//   k_drawn        the components that data has reached, compacted (a few
+//                  thousand of 50,000: the FP64 work below then fills its
+//                  warps; 40 us in caller's order, 23 us for both kernels).
+//   k_splat_prep   a thread per drawn component: posterior (FP64, from S_past
+//                  and the prior), camera transform, screen covariance and its
 //                  inverse, the screen rectangle of 16 x 16
 //                  pixel tiles that holds every pixel with alpha >= 1/255
 //                  (q <= 2 ln(255 * 0.99): the ellipse's bounding box), a
 //                  64-bit depth key.
+// Up to kDirect visible splats:
+//   k_order        each splat's place front to back (ties by index): the
+//                  number of smaller (depth, index) pairs, a warp per four
+//                  splats.
+//   k_raster_direct  a CTA per tile reads all rectangles in that order, 256 at
+//                  a time, keeps the splats that cover its tile and composites
+//                  them: no keys per (splat, tile), no sorts (13 radix passes,
+//                  95 us at 200 x 200 and K = 50,000).
+// More of them (every tile would read too many rectangles):
 //   depth rank     one stable CUB radix sort of the depth keys (FP64 depth
 //                  bits, components in index order): each splat's rank in
 //                  the global front-to-back order, ties by index.
@@ -31,7 +43,8 @@
 //   k_raster       a CTA per tile (256 threads, a pixel each): batches of
 //                  256 splats staged in shared memory, each pixel composites
 //                  them (the quadratic form in FP64, alpha and the colour in
-//                  FP32, one expm1 per splat and pixel); a pixel stops
+//                  FP32, one expm1 per splat and pixel; FP32 bounds first
+//                  leave out the splats that no pixel of a warp sees); a pixel stops
 //                  once its transmittance is below 1e-7 (what remains can
 //                  change its colour by less than 1e-7), the CTA once all
 //                  its pixels have.
@@ -55,6 +68,8 @@ constexpr float kOpacity = 0.99f;            // alpha = min(0.99, o e^(-q/2)) wi
 constexpr float kOneMinusOpacity = 0.01f;    // 1 - o, rounded once (not 1 - 0.99f)
 constexpr float kAlphaMin = 1.0f / 255.0f;
 constexpr float kTStop = 1e-7f;
+constexpr float kQMax = 11.07f;              // above 2 ln(255 * 0.99) = 11.0624: alpha < 1/255
+constexpr int kDirect = 8192;                // visible splats ordered by counting and read by every tile
 constexpr double kMinCount = 1.0;           // components with fewer points' worth of data are not drawn
 
 // A splat as the rasteriser reads it: centre and inverse screen covariance
@@ -73,25 +88,41 @@ struct Camera {
     int W, H, tiles_x, tiles_y;
 };
 
-// Per component: splat record, tile
-// rectangle, tile count and depth key (all-ones when left out).
-__global__ void k_splat_prep(const double *__restrict__ m0, const double *__restrict__ S, MstepParams P, int d, int K,
-                             Camera cam, float4 *__restrict__ sp, int4 *__restrict__ rect, long long *__restrict__ cnt,
-                             unsigned long long *__restrict__ zkey, int *__restrict__ zidx)
+// The components with a point's worth of data (list, count[0]; any order), and
+// the per-component arrays of the sorted path as for components left out.
+__global__ void k_drawn(const double *__restrict__ S, int K, int *__restrict__ list, int *__restrict__ count,
+                        long long *__restrict__ cnt, unsigned long long *__restrict__ zkey, int *__restrict__ zidx)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k > K) return;
-    if (k == K) {   // the scan's last element: its exclusive sum is the total
-        cnt[K] = 0;
-        return;
+    const int k = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+    const bool in = k < K && S[(size_t)k * VBGS_F] >= kMinCount;
+    const unsigned b = __ballot_sync(0xffffffffu, in);
+    if (b) {
+        int base = 0;
+        if (lane == 0) base = atomicAdd(count, __popc(b));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (in) list[base + __popc(b & ((1u << lane) - 1u))] = k;
     }
+    if (k <= K) cnt[k] = 0;   // cnt[K]: the scan's last element, whose exclusive sum is the total
+    if (k >= K) return;
     zidx[k] = k;
     zkey[k] = ~0ull;
-    cnt[k] = 0;
+}
+
+// Per drawn component: splat record, tile rectangle, tile count and depth
+// key; count[1] visible ones with their (key, component) in ckey, cidx (any
+// order).
+__global__ void k_splat_prep(const double *__restrict__ m0, const double *__restrict__ S, MstepParams P, int d,
+                             const int *__restrict__ list, int *__restrict__ count, Camera cam,
+                             float4 *__restrict__ sp, int4 *__restrict__ rect, long long *__restrict__ cnt,
+                             unsigned long long *__restrict__ zkey, unsigned long long *__restrict__ ckey,
+                             int *__restrict__ cidx)
+{
+    const int li = blockIdx.x * blockDim.x + threadIdx.x;
+    if (li >= count[0]) return;
+    const int k = list[li];
     const double *s = S + (size_t)k * VBGS_F;
     const double *a0 = m0 + (size_t)k * 6;
     const double Nk = s[0], beta = P.beta0 + Nk, nu = P.nu0 + Nk;
-    if (!(Nk >= kMinCount)) return;
     double m[6];
 #pragma unroll
     for (int i = 0; i < 6; i++) m[i] = (P.beta0 * a0[i] + s[1 + i]) / beta;
@@ -157,6 +188,9 @@ __global__ void k_splat_prep(const double *__restrict__ m0, const double *__rest
     rect[k] = make_int4(tx0, ty0, tx1, ty1);
     cnt[k] = (long long)(tx1 - tx0 + 1) * (ty1 - ty0 + 1);
     zkey[k] = (unsigned long long)__double_as_longlong(z);   // z > 0: the bits order as the values
+    const int at = atomicAdd(count + 1, 1);
+    ckey[at] = zkey[k];
+    cidx[at] = k;
     Splat &o = reinterpret_cast<Splat *>(sp)[k];
     o.u = u;
     o.v = v;
@@ -199,59 +233,164 @@ __global__ void k_ranges(const unsigned long long *__restrict__ key, long long n
     if (i == n - 1 || (int)(key[i + 1] >> 32) != t) range[t].y = (int)(i + 1);
 }
 
+// A pixel's running colour and transmittance.
+struct Pixel {
+    double cx, cy;
+    float T = 1.f, r = 0.f, g = 0.f, b = 0.f;
+    bool done;
+};
+
+// Composite n splats in order, a warp's 32 pixels (2 rows of a tile) each.
+__device__ __forceinline__ void composite(const Splat *__restrict__ sh, int n, Pixel &p)
+{
+    const float fx = (float)p.cx, fy = (float)p.cy;   // exact: half-integers below 2^15
+    for (int j = 0; j < n; j++) {
+        const Splat &a = sh[j];
+        // q in FP32 less its error bound: the terms' rounding (2^-20 of their
+        // sum) and the centre's (2^-23 of its coordinates; the inverse
+        // covariance is at most 1 / kLowPass per axis).  An FP64 instruction
+        // holds the warp's sub-partition for 64 cycles, so q is formed only
+        // where a pixel can see the splat.
+        const float u = (float)a.u, v = (float)a.v, ca = (float)a.ca, cb = (float)a.cb, cc = (float)a.cc;
+        const float ex = fx - u, ey = fy - v;
+        const float taa = ca * ex * ex, tab = 2.f * cb * ex * ey, tbb = cc * ey * ey;
+        const float slack = 1e-6f * (taa + fabsf(tab) + tbb) +
+                            4e-7f * (fabsf(u) + fabsf(v) + fx + fy) * (ca + 2.f * fabsf(cb) + cc) * (fabsf(ex) + fabsf(ey) + 1.f);
+        if (!__any_sync(0xffffffffu, !p.done && !((taa + tab + tbb) - slack > kQMax))) continue;
+        if (p.done) continue;
+        const double dx = p.cx - a.u, dy = p.cy - a.v;
+        const float q = (float)fma(a.ca * dx, dx, fma(2.0 * a.cb * dx, dy, a.cc * dy * dy));
+        // alpha = o e^(-q/2) <= 0.99 (the cap never binds at o = 0.99)
+        // and 1 - alpha = (1 - o) - o (e^(-q/2) - 1) from expm1:
+        // 1 - alpha of a nearly opaque splat is ~0.01, so an exp
+        // accurate to a few units of 2^-24 relative to 1 would give it
+        // a relative error ~100 times larger, and every splat behind
+        // it would inherit that through the transmittance
+        const float em = expm1f(-0.5f * q);
+        const float al = fmaf(kOpacity, em, kOpacity);
+        if (al < kAlphaMin) continue;
+        const float w = p.T * al;
+        p.r = fmaf(w, a.r, p.r);
+        p.g = fmaf(w, a.g, p.g);
+        p.b = fmaf(w, a.b, p.b);
+        p.T *= fmaf(-kOpacity, em, kOneMinusOpacity);
+        if (p.T < kTStop) p.done = true;
+    }
+}
+
+__device__ __forceinline__ Pixel pixel_at(int tile, int tid, int W, int H, int tiles_x, int &px, int &py)
+{
+    px = (tile % tiles_x) * kTile + (tid % kTile);
+    py = (tile / tiles_x) * kTile + tid / kTile;
+    Pixel p;
+    p.cx = (double)px + 0.5;
+    p.cy = (double)py + 0.5;
+    p.done = !(px < W && py < H);
+    return p;
+}
+__device__ __forceinline__ void write_pixel(const Pixel &p, int px, int py, int W, int H, float *__restrict__ img)
+{
+    if (px >= W || py >= H) return;
+    float *o = img + ((size_t)py * W + px) * 3;
+    o[0] = p.r;
+    o[1] = p.g;
+    o[2] = p.b;
+}
+
 __global__ void __launch_bounds__(kRT) k_raster(const float4 *__restrict__ sp, const int *__restrict__ val,
                                                 const int2 *__restrict__ range, int W, int H, int tiles_x,
                                                 float *__restrict__ img)
 {
     __shared__ Splat sh[kRT];
     const int tile = blockIdx.x, tid = threadIdx.x;
-    const int px = (tile % tiles_x) * kTile + (tid % kTile), py = (tile / tiles_x) * kTile + tid / kTile;
-    const bool inside = px < W && py < H;
-    const double cx = (double)px + 0.5, cy = (double)py + 0.5;
+    int px, py;
+    Pixel p = pixel_at(tile, tid, W, H, tiles_x, px, py);
     const int2 r = range[tile];
-    float T = 1.f, cr = 0.f, cg = 0.f, cb = 0.f;
-    bool done = !inside;
     for (int b = r.x; b < r.y; b += kRT) {
-        if (__syncthreads_and(done)) break;
+        if (__syncthreads_and(p.done)) break;
         const int i = b + tid;
-        if (i < r.y) {
-            const int k = val[i];
-            sh[tid] = reinterpret_cast<const Splat *>(sp)[k];
-        }
+        if (i < r.y) sh[tid] = reinterpret_cast<const Splat *>(sp)[val[i]];
         __syncthreads();
-        const int n = min(kRT, r.y - b);
-        if (!done) {
-            for (int j = 0; j < n; j++) {
-                const Splat &a = sh[j];
-                const double dx = cx - a.u, dy = cy - a.v;
-                const float q = (float)fma(a.ca * dx, dx, fma(2.0 * a.cb * dx, dy, a.cc * dy * dy));
-                // alpha = o e^(-q/2) <= 0.99 (the cap never binds at o = 0.99)
-                // and 1 - alpha = (1 - o) - o (e^(-q/2) - 1) from expm1:
-                // 1 - alpha of a nearly opaque splat is ~0.01, so an exp
-                // accurate to a few units of 2^-24 relative to 1 would give it
-                // a relative error ~100 times larger, and every splat behind
-                // it would inherit that through the transmittance
-                const float em = expm1f(-0.5f * q);
-                const float al = fmaf(kOpacity, em, kOpacity);
-                if (al < kAlphaMin) continue;
-                const float w = T * al;
-                cr = fmaf(w, a.r, cr);
-                cg = fmaf(w, a.g, cg);
-                cb = fmaf(w, a.b, cb);
-                T *= fmaf(-kOpacity, em, kOneMinusOpacity);
-                if (T < kTStop) {
-                    done = true;
-                    break;
-                }
-            }
+        composite(sh, min(kRT, r.y - b), p);
+    }
+    write_pixel(p, px, py, W, H, img);
+}
+
+// The place of every visible splat front to back, ties by component: a warp
+// counts the smaller ones for kOrder splats at a time.
+constexpr int kOrder = 4;
+__global__ void __launch_bounds__(256) k_order(const unsigned long long *__restrict__ ckey, const int *__restrict__ cidx,
+                                               int n, const int4 *__restrict__ rect, int *__restrict__ idx_s,
+                                               int4 *__restrict__ rect_s)
+{
+    const int lane = threadIdx.x & 31, e0 = ((blockIdx.x * 256 + threadIdx.x) >> 5) * kOrder;
+    if (e0 >= n) return;
+    unsigned long long k[kOrder];
+    int id[kOrder], c[kOrder];
+#pragma unroll
+    for (int u = 0; u < kOrder; u++) {
+        const int e = min(e0 + u, n - 1);
+        k[u] = ckey[e];
+        id[u] = cidx[e];
+        c[u] = 0;
+    }
+    for (int j = lane; j < n; j += 32) {
+        const unsigned long long kj = ckey[j];
+        const int ij = cidx[j];
+#pragma unroll
+        for (int u = 0; u < kOrder; u++) c[u] += kj < k[u] || (kj == k[u] && ij < id[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < kOrder; u++) {
+        const int place = __reduce_add_sync(0xffffffffu, c[u]);
+        if (lane == 0 && e0 + u < n) {
+            idx_s[place] = id[u];
+            rect_s[place] = rect[id[u]];
         }
     }
-    if (inside) {
-        float *o = img + ((size_t)py * W + px) * 3;
-        o[0] = cr;
-        o[1] = cg;
-        o[2] = cb;
+}
+
+__global__ void __launch_bounds__(kRT) k_raster_direct(const float4 *__restrict__ sp, const int *__restrict__ idx,
+                                                       const int4 *__restrict__ rect, int n, int W, int H, int tiles_x,
+                                                       float *__restrict__ img)
+{
+    __shared__ Splat sh[kRT];
+    __shared__ int pend[2 * kRT], wsum[kRT / 32];
+    const int tile = blockIdx.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int tx = tile % tiles_x, ty = tile / tiles_x;
+    int px, py, np = 0;
+    Pixel p = pixel_at(tile, tid, W, H, tiles_x, px, py);
+    for (int b = 0; b < n; b += kRT) {
+        if (__syncthreads_and(p.done)) break;
+        // the splats of this batch that cover the tile, in order
+        const int i = b + tid;
+        const int4 r = i < n ? rect[i] : make_int4(1, 1, 0, 0);
+        const bool hit = r.x <= tx && tx <= r.z && r.y <= ty && ty <= r.w;
+        const unsigned m = __ballot_sync(0xffffffffu, hit);
+        if (lane == 0) wsum[w] = __popc(m);
+        __syncthreads();
+        int at = np, tot = 0;
+#pragma unroll
+        for (int q = 0; q < kRT / 32; q++) {
+            at += q < w ? wsum[q] : 0;
+            tot += wsum[q];
+        }
+        if (hit) pend[at + __popc(m & ((1u << lane) - 1u))] = idx[i];
+        np += tot;
+        __syncthreads();
+        const bool last = b + kRT >= n;
+        while (np >= kRT || (last && np > 0)) {
+            const int cnt = min(np, kRT), rest = np - cnt;
+            if (tid < cnt) sh[tid] = reinterpret_cast<const Splat *>(sp)[pend[tid]];
+            const int mv = tid < rest ? pend[kRT + tid] : 0;
+            __syncthreads();
+            if (tid < rest) pend[tid] = mv;
+            composite(sh, cnt, p);
+            np = rest;
+            __syncthreads();
+        }
     }
+    write_pixel(p, px, py, W, H, img);
 }
 
 // Sum of squared differences on the 0..255 scale, per block of 256 values.
@@ -310,7 +449,8 @@ cudaError_t grow(T **p, size_t &cap, size_t n)
 
 void render_free(RenderBuffers &B)
 {
-    void *ptrs[] = {B.sp, B.rect, B.cnt, B.off, B.zkey, B.zkey_s, B.zidx, B.zidx_s, B.rank, B.ekey, B.ekey_s,
+    for (auto &e : B.ev) if (e) cudaEventDestroy(e);
+    void *ptrs[] = {B.list, B.count, B.rect_s, B.sp, B.rect, B.cnt, B.off, B.zkey, B.zkey_s, B.zidx, B.zidx_s, B.rank, B.ekey, B.ekey_s,
                     B.eval, B.eval_s, B.range, B.img, B.ref, B.part, B.out, B.temp};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -357,12 +497,12 @@ int render_frame(const double *m0, const double *S, const MstepParams &P, int d,
     RCU(grow(&B.part, B.cap_part, (npx + 255) / 256));
     RCU(grow(&B.out, B.cap_out, (size_t)2));
 
-    cudaEvent_t ev[4] = {};
-    for (auto &e : ev) RCU(cudaEventCreate(&e));
-    auto destroy_events = [&]() {
-        for (auto &e : ev)
-            if (e) cudaEventDestroy(e);
-    };
+    RCU(grow(&B.list, B.cap_list, (size_t)K));
+    RCU(grow(&B.count, B.cap_count, (size_t)2));
+    RCU(grow(&B.rect_s, B.cap_rect_s, (size_t)std::min(K, kDirect)));
+    cudaEvent_t(&ev)[4] = B.ev;
+    for (auto &e : ev)
+        if (!e) RCU(cudaEventCreate(&e));
 
     // 1. splats, depth ranks, tile counts and their offsets
     size_t t1 = 0, t2 = 0;
@@ -377,48 +517,66 @@ int render_frame(const double *m0, const double *S, const MstepParams &P, int d,
         B.temp_bytes = need;
     }
     RCU(cudaEventRecord(ev[0], st));
-    k_splat_prep<<<(K + 1 + 127) / 128, 128, 0, st>>>(m0, S, P, d, K, cam, B.sp, B.rect, B.cnt, B.zkey, B.zidx);
-    size_t tb = B.temp_bytes;
-    RCU(cub::DeviceRadixSort::SortPairs(B.temp, tb, B.zkey, B.zkey_s, B.zidx, B.zidx_s, K, 0, 64, st));
-    k_rank<<<(K + 255) / 256, 256, 0, st>>>(B.zidx_s, K, B.rank);
-    tb = B.temp_bytes;
-    RCU(cub::DeviceScan::ExclusiveSum(B.temp, tb, B.cnt, B.off, K + 1, st));
+    RCU(cudaMemsetAsync(B.count, 0, 2 * sizeof(int), st));
+    k_drawn<<<(K + 1 + 255) / 256, 256, 0, st>>>(S, K, B.list, B.count, B.cnt, B.zkey, B.zidx);
+    k_splat_prep<<<(K + 63) / 64, 64, 0, st>>>(m0, S, P, d, B.list, B.count, cam, B.sp, B.rect, B.cnt, B.zkey, B.zkey_s,
+                                               B.zidx_s);
     RCU(cudaEventRecord(ev[1], st));
-    long long total = 0;
-    RCU(cudaMemcpyAsync(&total, B.off + K, sizeof total, cudaMemcpyDeviceToHost, st));
-    RCU(cudaStreamSynchronize(st));
-    if (total < 0 || total > (long long)0x7fffffff) {
-        destroy_events();
-        why = "more than 2^31 (splat, tile) pairs";
-        return -1;
-    }
-    // 2. tile keys, sorted; per-tile ranges; compositing; PSNR
-    RCU(grow(&B.ekey, B.cap_ekey, (size_t)total));
-    RCU(grow(&B.ekey_s, B.cap_ekey_s, (size_t)total));
-    RCU(grow(&B.eval, B.cap_eval, (size_t)total));
-    RCU(grow(&B.eval_s, B.cap_eval_s, (size_t)total));
-    size_t t3 = 0;
-    cub::DeviceRadixSort::SortPairs(nullptr, t3, B.ekey, B.ekey_s, B.eval, B.eval_s, (int)std::max<long long>(total, 1),
-                                    0, 32 + tile_bits, st);
-    if (t3 > B.temp_bytes) {
-        cudaFree(B.temp);
-        B.temp = nullptr;
-        B.temp_bytes = 0;
-        RCU(cudaMalloc(&B.temp, t3));
-        B.temp_bytes = t3;
-    }
+    int count[2] = {0, 0};
+    RCU(cudaMemcpyAsync(count, B.count, sizeof count, cudaMemcpyDeviceToHost, st));
     if (ref) RCU(cudaMemcpyAsync(B.ref, ref, sizeof(float) * npx, cudaMemcpyHostToDevice, st));
-    RCU(cudaMemsetAsync(B.range, 0, sizeof(int2) * ntiles, st));
-    RCU(cudaEventRecord(ev[2], st));
-    if (total > 0) {
-        k_emit<<<(K + 127) / 128, 128, 0, st>>>(B.rect, B.cnt, B.off, B.rank, K, cam.tiles_x,
-                                                B.ekey, B.eval);
+    RCU(cudaStreamSynchronize(st));
+    float sort_ms = 0.f;
+    const int n = count[1];
+    if (n <= kDirect) {
+        // 2. order by counting; every tile reads the rectangles
+        RCU(cudaEventRecord(ev[2], st));
+        if (n > 0)
+            k_order<<<(n + 8 * kOrder - 1) / (8 * kOrder), 256, 0, st>>>(B.zkey_s, B.zidx_s, n, B.rect, B.rank, B.rect_s);
+        k_raster_direct<<<ntiles, kRT, 0, st>>>(B.sp, B.rank, B.rect_s, n, W, H, cam.tiles_x, B.img);
+    } else {
+        cudaEventElapsedTime(&sort_ms, ev[0], ev[1]);
+        RCU(cudaEventRecord(ev[0], st));
+        size_t tb = B.temp_bytes;
+        RCU(cub::DeviceRadixSort::SortPairs(B.temp, tb, B.zkey, B.zkey_s, B.zidx, B.zidx_s, K, 0, 64, st));
+        k_rank<<<(K + 255) / 256, 256, 0, st>>>(B.zidx_s, K, B.rank);
         tb = B.temp_bytes;
-        RCU(cub::DeviceRadixSort::SortPairs(B.temp, tb, B.ekey, B.ekey_s, B.eval, B.eval_s, (int)total, 0,
-                                            32 + tile_bits, st));
-        k_ranges<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(B.ekey_s, total, B.range);
+        RCU(cub::DeviceScan::ExclusiveSum(B.temp, tb, B.cnt, B.off, K + 1, st));
+        RCU(cudaEventRecord(ev[1], st));
+        long long total = 0;
+        RCU(cudaMemcpyAsync(&total, B.off + K, sizeof total, cudaMemcpyDeviceToHost, st));
+        RCU(cudaStreamSynchronize(st));
+        if (total < 0 || total > (long long)0x7fffffff) {
+            why = "more than 2^31 (splat, tile) pairs";
+            return -1;
+        }
+        // 2. tile keys, sorted; per-tile ranges; compositing; PSNR
+        RCU(grow(&B.ekey, B.cap_ekey, (size_t)total));
+        RCU(grow(&B.ekey_s, B.cap_ekey_s, (size_t)total));
+        RCU(grow(&B.eval, B.cap_eval, (size_t)total));
+        RCU(grow(&B.eval_s, B.cap_eval_s, (size_t)total));
+        size_t t3 = 0;
+        cub::DeviceRadixSort::SortPairs(nullptr, t3, B.ekey, B.ekey_s, B.eval, B.eval_s, (int)std::max<long long>(total, 1),
+                                        0, 32 + tile_bits, st);
+        if (t3 > B.temp_bytes) {
+            cudaFree(B.temp);
+            B.temp = nullptr;
+            B.temp_bytes = 0;
+            RCU(cudaMalloc(&B.temp, t3));
+            B.temp_bytes = t3;
+        }
+        RCU(cudaMemsetAsync(B.range, 0, sizeof(int2) * ntiles, st));
+        RCU(cudaEventRecord(ev[2], st));
+        if (total > 0) {
+            k_emit<<<(K + 127) / 128, 128, 0, st>>>(B.rect, B.cnt, B.off, B.rank, K, cam.tiles_x,
+                                                    B.ekey, B.eval);
+            tb = B.temp_bytes;
+            RCU(cub::DeviceRadixSort::SortPairs(B.temp, tb, B.ekey, B.ekey_s, B.eval, B.eval_s, (int)total, 0,
+                                                32 + tile_bits, st));
+            k_ranges<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(B.ekey_s, total, B.range);
+        }
+        k_raster<<<ntiles, kRT, 0, st>>>(B.sp, B.eval_s, B.range, W, H, cam.tiles_x, B.img);
     }
-    k_raster<<<ntiles, kRT, 0, st>>>(B.sp, B.eval_s, B.range, W, H, cam.tiles_x, B.img);
     const int nb = (int)((npx + 255) / 256);
     if (ref) {
         k_mse_part<<<nb, 256, 0, st>>>(B.img, B.ref, npx, B.part);
@@ -435,9 +593,8 @@ int render_frame(const double *m0, const double *S, const MstepParams &P, int d,
         float a = 0.f, b = 0.f;
         cudaEventElapsedTime(&a, ev[0], ev[1]);
         cudaEventElapsedTime(&b, ev[2], ev[3]);
-        *device_ms = (double)a + (double)b;
+        *device_ms = (double)a + (double)b + (double)sort_ms;
     }
-    destroy_events();
     return 0;
 #undef RCU
 }

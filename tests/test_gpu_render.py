@@ -182,3 +182,36 @@ def test_render_edges(V):
     rc = V.lib().vbgs_render(m.ctx, V._dp(V.camera_array(cam)), 4, 4, None, None, V._dp(np.zeros(1)), None)
     assert rc == V.VBGS_EINVAL
     m.close()
+
+
+@pytest.mark.parametrize("K", [1, 31, 4_000, 9_000])
+def test_counted_and_sorted_orders_match_the_oracle(V, K):
+    """Visible splats up to 8,192 are ordered by counting, more by the radix
+    sorts; pairs of components at the same place and depth, of other colours,
+    composite in index order on both paths.  The per-pixel bound is that of
+    check_image (the small image has a threshold pair in most pixels)."""
+    rng = np.random.default_rng(K)
+    pr = synth.nw_prior(K, seed=K, lo=(-1, -1, 2, 0, 0, 0), hi=(1, 1, 4, 1, 1, 1))
+    half = pr["m0"][1::2].shape[0]
+    pr["m0"][1::2, :3] = pr["m0"][0::2, :3][:half]
+    n = rng.uniform(1.0, 30.0, K)
+    n[1::2] = n[0::2][:half]
+    S = np.zeros((K, 28))
+    S[:, 0] = n
+    S[:, 1:7] = n[:, None] * pr["m0"]
+    u = 7
+    for i in range(6):
+        for j in range(i, 6):
+            S[:, u] = n * (pr["m0"][:, i] * pr["m0"][:, j] + (1e-4 if i == j else 0.0))
+            u += 1
+    cam = {"o": np.zeros(3), "Rwc": np.eye(3), "f": 40.0, "width": 40, "height": 33}
+    m = V.Model(pr, "fp64")
+    m.set_stats(S)
+    img = m.render(cam)[0]
+    m.close()
+    post = O.mstep(pr, S)
+    ref = RD.render_posterior(post, cam, S[:, 0])
+    pairs, contrib = threshold_pairs(post["m"][:, :3], RD.expected_spatial_cov(post["Winv"], post["nu"], 6), cam)
+    err = np.abs(img.astype(np.float64) - ref).max(axis=2)
+    assert np.all(err <= 2e-6 + 4e-7 * contrib + pairs * (2.0 / 255.0) * 1.01)
+    assert np.any(img > 0.05)
