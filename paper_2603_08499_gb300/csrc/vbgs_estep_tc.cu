@@ -30,6 +30,7 @@
 // (8-row group) stride 512 B.  Coefficient tiles are built in global memory
 // in exactly this layout so one bulk copy stages them.
 #include "vbgs_internal.cuh"
+#include "vbgs_pair.cuh"
 #include "vbgs_tc.cuh"
 #include <cuda_fp16.h>
 #include <cuda_bf16.h>
@@ -210,19 +211,6 @@ __device__ __forceinline__ dfl df_from_bits(double v)
     const float scale = __uint_as_float((unsigned)(ex - 1075 + 127) << 23);   // 2^(ex - 1075), a normal float
     const float l = __uint2float_rn((unsigned)(b & 0x1fffffffu)) * scale;
     return {h, sgn ? -l : l};
-}
-// FP32 -> FP64 without an FP64 instruction: the exponent rebiased and the
-// significand widened, exact for zeros and normal numbers; subnormals,
-// infinities and NaNs take the conversion instruction.
-__device__ __forceinline__ double f2d_exact(float f)
-{
-    const unsigned b = __float_as_uint(f);
-    const unsigned ex = (b >> 23) & 0xffu;
-    const unsigned long long sgn = (unsigned long long)(b & 0x80000000u) << 32;
-    if ((b << 1) == 0u) return __longlong_as_double((long long)sgn);
-    if (ex == 0u || ex == 0xffu) return (double)f;
-    return __longlong_as_double((long long)(sgn | ((unsigned long long)(ex + 896u) << 52) |
-                                            ((unsigned long long)(b & 0x7fffffu) << 29)));
 }
 // sqrt(log2 e) and log2 e as double-float pairs
 constexpr float kS2h = 1.2011224031448364f, kS2l = 5.641613398665868e-09f;

@@ -1,6 +1,6 @@
 // vbgs_pair.cuh -- the logit of one (point, component) pair on the CUDA cores,
 // shared by the dense passes (vbgs_estep_cc.cu) and the sparse ones
-// (vbgs_estep_sparse.cu).
+// (vbgs_estep_sparse.cu), and an exact FP32 -> FP64 conversion.
 #pragma once
 #include "vbgs_internal.cuh"
 
@@ -76,4 +76,17 @@ __device__ __forceinline__ float quad_rest(const float *__restrict__ r, const fl
     return q;
 }
 
+// FP32 -> FP64 without an FP64 instruction: the exponent rebiased and the
+// significand widened, exact for zeros and normal numbers; subnormals,
+// infinities and NaNs take the conversion instruction.
+__device__ __forceinline__ double f2d_exact(float f)
+{
+    const unsigned b = __float_as_uint(f);
+    const unsigned ex = (b >> 23) & 0xffu;
+    const unsigned long long sgn = (unsigned long long)(b & 0x80000000u) << 32;
+    if ((b << 1) == 0u) return __longlong_as_double((long long)sgn);
+    if (ex == 0u || ex == 0xffu) return (double)f;
+    return __longlong_as_double((long long)(sgn | ((unsigned long long)(ex + 896u) << 52) |
+                                            ((unsigned long long)(b & 0x7fffffu) << 29)));
+}
 } // namespace vbgs

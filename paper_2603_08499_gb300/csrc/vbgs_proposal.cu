@@ -18,6 +18,7 @@
 // and, like every E-step logit of the library, without the -psi(sum alpha)
 // term shared by all components (it cancels in every ratio used here).
 #include "vbgs_internal.cuh"
+#include "vbgs_pair.cuh"
 #include <cub/device/device_radix_sort.cuh>
 #include <algorithm>
 
@@ -64,31 +65,55 @@ __global__ void k_means_of_records(const float *__restrict__ rec32, int K, float
     for (int i = 0; i < 6; i++) pts[(size_t)p * 6 + i] = rec32[(size_t)p * VBGS_REC + i] * (i < 3 ? 1.f : csc);
 }
 
-// Nearest centroid (squared distance in FP32, ties to the lower index).
-__global__ void __launch_bounds__(256) k_assign(const float *__restrict__ pts, int K, const float *__restrict__ cent,
-                                                unsigned int *__restrict__ key, int *__restrict__ idx)
+// Nearest centroid (squared distance in FP32, ties to the lower index), two
+// points a thread: the differences and squares of both in paired FP32
+// arithmetic (each half rounded like the scalar instruction), the centroids
+// negated and duplicated in shared memory so that a pair costs three vector
+// loads and 12 instructions for 24 scalar ones.  Bound by instruction issue:
+// K = 200,000 x 1,024: 120 -> 100 us.
+__device__ __forceinline__ unsigned long long pair2(float a, float b)
 {
-    __shared__ float sc[kG * 6];
-    for (int i = threadIdx.x; i < kG * 6; i += blockDim.x) sc[i] = cent[i];
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+constexpr int kAssign = 128;   // threads
+__global__ void __launch_bounds__(kAssign) k_assign(const float *__restrict__ pts, int K, const float *__restrict__ cent,
+                                                    unsigned int *__restrict__ key, int *__restrict__ idx)
+{
+    __shared__ __align__(16) unsigned long long sc[kG * 6];   // (-c, -c)
+    for (int i = threadIdx.x; i < kG * 6; i += kAssign) sc[i] = pair2(-cent[i], -cent[i]);
     __syncthreads();
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= K) return;
-    float x[6];
+    const int p0 = blockIdx.x * 2 * kAssign + threadIdx.x, p1 = p0 + kAssign;
+    if (p0 >= K) return;
+    unsigned long long x[6];
 #pragma unroll
-    for (int i = 0; i < 6; i++) x[i] = pts[(size_t)p * 6 + i];
-    float best = INFINITY;
-    int bg = 0;
+    for (int i = 0; i < 6; i++) x[i] = pair2(pts[(size_t)p0 * 6 + i], pts[(size_t)min(p1, K - 1) * 6 + i]);
+    float b0 = INFINITY, b1 = INFINITY;
+    int g0 = 0, g1 = 0;
+#pragma unroll 4
     for (int g = 0; g < kG; g++) {
-        float d2 = 0.f;
+        const ulonglong2 *c2 = reinterpret_cast<const ulonglong2 *>(sc + g * 6);
+        const ulonglong2 ca = c2[0], cb = c2[1], cc = c2[2];
+        const unsigned long long c[6] = {ca.x, ca.y, cb.x, cb.y, cc.x, cc.y};
+        unsigned long long d2 = 0ull;
 #pragma unroll
         for (int i = 0; i < 6; i++) {
-            const float t = x[i] - sc[g * 6 + i];
-            d2 = fmaf(t, t, d2);
+            unsigned long long t;
+            asm("add.rn.f32x2 %0, %1, %2;" : "=l"(t) : "l"(x[i]), "l"(c[i]));
+            asm("fma.rn.f32x2 %0, %1, %1, %2;" : "=l"(d2) : "l"(t), "l"(d2));
         }
-        if (d2 < best) { best = d2; bg = g; }
+        float e0, e1;
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(e0), "=f"(e1) : "l"(d2));
+        if (e0 < b0) { b0 = e0; g0 = g; }
+        if (e1 < b1) { b1 = e1; g1 = g; }
     }
-    key[p] = (unsigned int)bg;
-    idx[p] = p;
+    key[p0] = (unsigned int)g0;
+    idx[p0] = p0;
+    if (p1 < K) {
+        key[p1] = (unsigned int)g1;
+        idx[p1] = p1;
+    }
 }
 
 // Cluster boundaries of the sorted assignment (cstart[g] .. cstart[g+1]).
@@ -187,7 +212,7 @@ __device__ double lmax_bound6(const double *S)
     for (int i = 0; i < 6; i++)
 #pragma unroll
         for (int j = 0; j <= i; j++) f += (i == j ? 1.0 : 2.0) * (double)B[tri(i, j)] * (double)B[tri(i, j)];
-    return t * pow(sqrt(f), 0.125) * (1.0 + 1e-4);
+    return t * sqrt(sqrt(sqrt(sqrt(f)))) * (1.0 + 1e-4);   // f^(1/16)
 }
 
 // Cluster centre and metric: o = mean of the member means, P = the average
@@ -284,7 +309,9 @@ __device__ __forceinline__ float f_down(double v)
 }
 
 // Per member (sorted position i): constant (log2, rounded up), the four
-// scales mu (rounded down) and the four radii r (rounded up).
+// scales mu (rounded down) and the four radii r (rounded up).  Bound by the
+// FP64 pipe: with a reciprocal per row instead of a division per entry and
+// square roots for f^(1/16), 381 -> 273 us at K = 200,000.
 __global__ void __launch_bounds__(128) k_cluster_members(const double *__restrict__ rec,
                                                          const float *__restrict__ rec32,
                                                          const int *__restrict__ order,
@@ -298,21 +325,29 @@ __global__ void __launch_bounds__(128) k_cluster_members(const double *__restric
     const double *r = rec + (size_t)p * VBGS_REC;
     const double *cs = cscr + (size_t)g * kCScr;
     double M[21], Mi[21];
+#pragma unroll
     for (int q = 0; q < 21; q++) M[q] = r[6 + q];
-    // inverse of the lower-triangular M
-    for (int j = 0; j < 6; j++) {
-        Mi[tri(j, j)] = 1.0 / M[tri(j, j)];
+    // inverse of the lower-triangular M (six reciprocals: an FP64 division is
+    // about ten instructions of 64 cycles)
+#pragma unroll
+    for (int j = 0; j < 6; j++) Mi[tri(j, j)] = 1.0 / M[tri(j, j)];
+#pragma unroll
+    for (int j = 0; j < 6; j++)
+#pragma unroll
         for (int a = j + 1; a < 6; a++) {
             double v = 0.0;
+#pragma unroll
             for (int l = j; l < a; l++) v = fma(M[tri(a, l)], Mi[tri(l, j)], v);
-            Mi[tri(a, j)] = -v / M[tri(a, a)];
+            Mi[tri(a, j)] = -v * Mi[tri(a, a)];
         }
-    }
     // covariance Sigma = Lam^-1 = Mi Mi^T
     double Sg[21];
+#pragma unroll
     for (int a = 0; a < 6; a++)
+#pragma unroll
         for (int c = 0; c <= a; c++) {
             double v = 0.0;
+#pragma unroll
             for (int l = 0; l <= c; l++) v = fma(Mi[tri(a, l)], Mi[tri(c, l)], v);
             Sg[tri(a, c)] = v;
         }
@@ -322,16 +357,22 @@ __global__ void __launch_bounds__(128) k_cluster_members(const double *__restric
     const double *L = cs + 6;
     if (cs[27] != 0.0) {
         double Z[36];   // Sigma L
+#pragma unroll
         for (int a = 0; a < 6; a++)
+#pragma unroll
             for (int c = 0; c < 6; c++) {
                 double v = 0.0;
+#pragma unroll
                 for (int l = c; l < 6; l++) v = fma(Sg[a >= l ? tri(a, l) : tri(l, a)], L[tri(l, c)], v);
                 Z[a * 6 + c] = v;
             }
         double A[21];   // L^T Sigma L
+#pragma unroll
         for (int a = 0; a < 6; a++)
+#pragma unroll
             for (int c = 0; c <= a; c++) {
                 double v = 0.0;
+#pragma unroll
                 for (int l = a; l < 6; l++) v = fma(L[tri(l, a)], Z[l * 6 + c], v);
                 A[tri(a, c)] = v;
             }
@@ -340,10 +381,14 @@ __global__ void __launch_bounds__(128) k_cluster_members(const double *__restric
     const double lp = (double)rec32[(size_t)p * VBGS_REC + 28] * 0.6931471805599453 * (1.0 - 1e-6);
     const double lc = (double)rec32[(size_t)p * VBGS_REC + 29] * 0.6931471805599453 * (1.0 - 1e-6);
     double dx[6], rp = 0.0, rc = 0.0, rm = 0.0;
+#pragma unroll
     for (int q = 0; q < 6; q++) dx[q] = r[q] - cs[q];
+#pragma unroll
     for (int q = 0; q < 3; q++) { rp = fma(dx[q], dx[q], rp); rc = fma(dx[3 + q], dx[3 + q], rc); }
+#pragma unroll
     for (int c = 0; c < 6; c++) {
         double y = 0.0;
+#pragma unroll
         for (int a = c; a < 6; a++) y = fma(L[tri(a, c)], dx[a], y);
         rm = fma(y, y, rm);
     }
@@ -731,7 +776,13 @@ __global__ void __launch_bounds__(kPB) k_cand_score(const double *__restrict__ X
         __syncthreads();
         if (live)
             for (int mm = 0; mm < ms; mm++) {
-                const float l = logit32(sr + mm * 28, x);
+                float r[28];   // seven vector loads, the same row in every lane
+#pragma unroll
+                for (int q = 0; q < 7; q++) {
+                    const float4 t4 = reinterpret_cast<const float4 *>(sr + mm * 28)[q];
+                    r[4 * q] = t4.x; r[4 * q + 1] = t4.y; r[4 * q + 2] = t4.z; r[4 * q + 3] = t4.w;
+                }
+                const float l = logit32(r, x);
                 if (l > mx) { sum = sum * ex2a(mx - l) + 1.f; mx = l; }
                 else sum += ex2a(l - mx);
             }
@@ -922,7 +973,11 @@ __global__ void __launch_bounds__(1024) k_items(const int *__restrict__ pstart, 
     if (g == 0) { item_start[0] = 0; fbase[0] = 0; }
 }
 
+// Candidate pass 2: a CTA per (work item of kPB2 points, slice of 64 of the
+// cluster's members), a thread per member.  One CTA for all members of an item
+// left the few large clusters' items running alone: 470 -> 349 us.
 constexpr int kPB2 = 512;   // points per work item of candidate pass 2
+constexpr int kMemberSlices = 8;
 
 __global__ void __launch_bounds__(64) k_cand_pass2(const double *__restrict__ X, const double *__restrict__ lse_c,
                                                    const float *__restrict__ rec32, const int *__restrict__ order,
@@ -930,7 +985,7 @@ __global__ void __launch_bounds__(64) k_cand_pass2(const double *__restrict__ X,
                                                    const int *__restrict__ plist, const int *__restrict__ item_start,
                                                    const long long *__restrict__ fbase, float *__restrict__ part)
 {
-    __shared__ float sp[kPB2][8];
+    __shared__ __align__(16) float sp[kPB2][8];
     __shared__ int sg;
     const int item = blockIdx.x;
     if (threadIdx.x == 0) {
@@ -946,6 +1001,7 @@ __global__ void __launch_bounds__(64) k_cand_pass2(const double *__restrict__ X,
     const int c = item - item_start[g];
     const int b = cstart[g], S = cstart[g + 1] - b;
     const int p0 = pstart[g] + c * kPB2, cnt = min(kPB2, pstart[g + 1] - p0);
+    if ((int)(blockIdx.y * blockDim.x) >= S) return;
     for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
         const int n = plist[p0 + t];
 #pragma unroll
@@ -953,7 +1009,7 @@ __global__ void __launch_bounds__(64) k_cand_pass2(const double *__restrict__ X,
         sp[t][6] = (float)(lse_c[n] * 1.4426950408889634);
     }
     __syncthreads();
-    for (int m0 = 0; m0 < S; m0 += blockDim.x) {
+    for (int m0 = blockIdx.y * blockDim.x; m0 < S; m0 += blockDim.x * gridDim.y) {
         const int ml = m0 + threadIdx.x;
         if (ml >= S) break;
         const int pos = order[b + ml];
@@ -964,10 +1020,9 @@ __global__ void __launch_bounds__(64) k_cand_pass2(const double *__restrict__ X,
 #pragma unroll
         for (int f = 0; f < 28; f++) acc[f] = 0.f;
         for (int t = 0; t < cnt; t++) {
-            float x[6];
-#pragma unroll
-            for (int q = 0; q < 6; q++) x[q] = sp[t][q];
-            const float w = ex2a(logit32(r, x) - sp[t][6]);
+            const float4 pa = reinterpret_cast<const float4 *>(sp[t])[0], pb = reinterpret_cast<const float4 *>(sp[t])[1];
+            const float x[6] = {pa.x, pa.y, pa.z, pa.w, pb.x, pb.y};
+            const float w = ex2a(logit32(r, x) - pb.z);
             acc[0] += w;
             float d[6], wd[6];
 #pragma unroll
@@ -984,7 +1039,7 @@ __global__ void __launch_bounds__(64) k_cand_pass2(const double *__restrict__ X,
     }
 }
 
-// One CTA per cluster: lane = member (32 at a time), warp w sums the items
+// A CTA per (cluster, slice of its members): lane = member (32 at a time), warp w sums the items
 // c = w, w + 4, ... in order; the four warp sums are added in warp order.
 __global__ void __launch_bounds__(128) k_cand_reduce(const float *__restrict__ part, const float *__restrict__ rec32,
                                                      const int *__restrict__ order, const int *__restrict__ cstart,
@@ -997,7 +1052,7 @@ __global__ void __launch_bounds__(128) k_cand_reduce(const float *__restrict__ p
     const int b = cstart[g], S = cstart[g + 1] - b;
     const int items = item_start[g + 1] - item_start[g];
     if (items == 0) return;
-    for (int m0 = 0; m0 < S; m0 += 32) {
+    for (int m0 = blockIdx.y * 32; m0 < S; m0 += 32 * gridDim.y) {
         const int ml = m0 + lane;
         const bool v = ml < S;
         double s[28];
@@ -1007,7 +1062,7 @@ __global__ void __launch_bounds__(128) k_cand_reduce(const float *__restrict__ p
             for (int c = w; c < items; c += 4) {
                 const float *src = part + (fbase[g] + (long long)c * S + ml) * VBGS_F;
 #pragma unroll
-                for (int f = 0; f < 28; f++) s[f] += (double)src[f];
+                for (int f = 0; f < 28; f++) s[f] += f2d_exact(src[f]);   // the sum alone is on the FP64 pipe
             }
         __syncthreads();
         if (w > 0)
@@ -1047,8 +1102,11 @@ __global__ void k_list_bounds(const unsigned int *__restrict__ skey, int64_t n, 
 
 // Labels of the exact points: q_ng = sum_{k in g} 2^(l_nk - lse2_n), over the
 // clusters whose certificate bound is not below 2^-40 of the point's mass
-// (UB row of the point's frame index: rows[i] when the points were gathered).  One warp
-// per point: lanes test the clusters, then share the scoring of each kept one.
+// (UB row of the point's frame index: rows[i] when the points were gathered).  A warp per
+// (point, slice of the clusters): lanes test the clusters, then share the
+// scoring of each kept one.  A few hundred points alone would hold a few
+// hundred warps: one warp a point 715 us, eight 173.
+constexpr int kLabelSlices = 8;
 __global__ void __launch_bounds__(256) k_labels(const double *__restrict__ Xe, const double *__restrict__ lse_e,
                                                 const int *__restrict__ rows, int64_t rstride, int64_t ne,
                                                 const float *__restrict__ rec32, const int *__restrict__ order,
@@ -1064,7 +1122,8 @@ __global__ void __launch_bounds__(256) k_labels(const double *__restrict__ Xe, c
     const float l2 = (float)(lse_e[n * rstride] * 1.4426950408889634);
     float *q = Q + deal_slot(n, nb, S) * kG;
     const float *ub = UB + (int64_t)(rows ? rows[n * rstride] : n * rstride) * kG;
-    for (int g0 = 0; g0 < kG; g0 += 32) {
+    const int gs = blockIdx.y * (kG / kLabelSlices);
+    for (int g0 = gs; g0 < gs + kG / kLabelSlices; g0 += 32) {
         const int g = g0 + lane;
         const bool keep = ub[g] - l2 > -40.f;
         if (!keep) q[g] = 0.f;
@@ -1074,8 +1133,16 @@ __global__ void __launch_bounds__(256) k_labels(const double *__restrict__ Xe, c
             kb &= kb - 1;
             const int gg = g0 + j;
             float v = 0.f;
-            for (int i = cstart[gg] + lane; i < cstart[gg + 1]; i += 32)
-                v += ex2a(logit32(rec32 + (size_t)order[i] * VBGS_REC, x) - l2);
+            for (int i = cstart[gg] + lane; i < cstart[gg + 1]; i += 32) {
+                const float4 *row = reinterpret_cast<const float4 *>(rec32 + (size_t)order[i] * VBGS_REC);
+                float r[28];   // a lane's own record: seven vector loads, not 28 strided ones
+#pragma unroll
+                for (int u = 0; u < 7; u++) {
+                    const float4 t4 = row[u];
+                    r[4 * u] = t4.x; r[4 * u + 1] = t4.y; r[4 * u + 2] = t4.z; r[4 * u + 3] = t4.w;
+                }
+                v += ex2a(logit32(r, x) - l2);
+            }
             v = warp_sum(v);
             if (lane == 0) q[gg] = v;
         }
@@ -1102,46 +1169,45 @@ __global__ void __launch_bounds__(256) k_audit_part(const double *__restrict__ X
                                                     int64_t ne, const int *__restrict__ exact,
                                                     const float *__restrict__ rec32, int K, float2 *__restrict__ part)
 {
-    __shared__ float xs[kAP][6];
-    __shared__ int live[kAP];
-    __shared__ float2 wp[kAP][8];
+    // lane = row; the block's 256 records in shared memory, a warp takes every
+    // eighth, so a pair costs no shuffle (lane = component, a warp reduction per
+    // row: 393 us, now 164)
+    __shared__ __align__(16) float sr[256 * 28];
+    __shared__ float2 wp[8][kAP];
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    const int64_t i0 = (int64_t)blockIdx.x * kAP;
-    if (t < kAP) {
-        const int64_t i = i0 + t;
-        const bool ok = i < ne && exact[erows[i]] == 2;
-        live[t] = ok;
+    const int64_t i = (int64_t)blockIdx.x * kAP + lane;
+    const int k0 = blockIdx.y * 256, cnt = min(256, K - k0);
+    const bool live = i < ne && exact[erows[i]] == 2;
+    float x[6];
 #pragma unroll
-        for (int q = 0; q < 6; q++) xs[t][q] = ok ? (float)X[(int64_t)erows[i] * VBGS_XS + q] : 0.f;
-    }
+    for (int q = 0; q < 6; q++) x[q] = live ? (float)X[(int64_t)erows[i] * VBGS_XS + q] : 0.f;
+    for (int j = t; j < cnt * 7; j += 256)
+        reinterpret_cast<float4 *>(sr)[j] = reinterpret_cast<const float4 *>(rec32 + (size_t)(k0 + j / 7) * VBGS_REC)[j % 7];
     __syncthreads();
-    const int k = blockIdx.y * 256 + t;
-    const bool kv = k < K;
-    float r[28];
+    float m = -INFINITY, sum = 0.f;
+    for (int k = w; k < cnt; k += 8) {
+        float r[28];
 #pragma unroll
-    for (int q = 0; q < 28; q++) r[q] = kv ? rec32[(size_t)k * VBGS_REC + q] : 0.f;
-    for (int p = 0; p < kAP; p++) {
-        if (!live[p]) continue;
-        float x[6];
-#pragma unroll
-        for (int q = 0; q < 6; q++) x[q] = xs[p][q];
-        const float l = kv ? logit32(r, x) : -INFINITY;
-        const float m = warp_max(l);
-        const float e = (m == -INFINITY) ? 0.f : warp_sum(ex2a(l - m));
-        if (lane == 0) wp[p][w] = make_float2(m, e);
-    }
-    __syncthreads();
-    if (t < kAP) {
-        float2 out = make_float2(-INFINITY, 0.f);
-        if (live[t]) {
-            float m = -INFINITY;
-            for (int q = 0; q < 8; q++) m = fmaxf(m, wp[t][q].x);
-            float sum = 0.f;
-            if (m != -INFINITY)
-                for (int q = 0; q < 8; q++) sum += wp[t][q].y * ex2a(wp[t][q].x - m);
-            out = make_float2(m, sum);
+        for (int q = 0; q < 7; q++) {
+            const float4 t4 = reinterpret_cast<const float4 *>(sr + k * 28)[q];
+            r[4 * q] = t4.x; r[4 * q + 1] = t4.y; r[4 * q + 2] = t4.z; r[4 * q + 3] = t4.w;
         }
-        if (i0 + t < ne) part[(i0 + t) * gridDim.y + blockIdx.y] = out;
+        const float l = logit32(r, x);
+        if (l > m) { sum = sum * ex2a(m - l) + 1.f; m = l; }
+        else sum += ex2a(l - m);
+    }
+    wp[w][lane] = make_float2(m, sum);
+    __syncthreads();
+    if (w == 0 && i < ne) {
+        float2 out = make_float2(-INFINITY, 0.f);
+        if (live) {
+            float mm = -INFINITY, ss = 0.f;
+            for (int q = 0; q < 8; q++) mm = fmaxf(mm, wp[q][lane].x);
+            if (mm != -INFINITY)
+                for (int q = 0; q < 8; q++) ss += wp[q][lane].y * ex2a(wp[q][lane].x - mm);
+            out = make_float2(mm, ss);
+        }
+        part[i * gridDim.y + blockIdx.y] = out;
     }
 }
 
@@ -1150,18 +1216,25 @@ __global__ void __launch_bounds__(256) k_audit_final(const float2 *__restrict__ 
                                                      const int *__restrict__ exact, const double *__restrict__ lse_c,
                                                      float *__restrict__ audit_missed)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31;
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;   // a warp per row
     if (i >= ne) return;
     const int n = erows[i];
-    if (exact[n] != 2) { audit_missed[i] = 0.f; return; }
+    if (exact[n] != 2) {
+        if (lane == 0) audit_missed[i] = 0.f;
+        return;
+    }
     float m = -INFINITY;
-    for (int c = 0; c < nch; c++) m = fmaxf(m, part[i * nch + c].x);
+    for (int c = lane; c < nch; c += 32) m = fmaxf(m, part[i * nch + c].x);
+    m = warp_max(m);
     double s = 0.0;
-    for (int c = 0; c < nch; c++)
+    for (int c = lane; c < nch; c += 32)
         if (part[i * nch + c].x != -INFINITY) s += (double)part[i * nch + c].y * (double)ex2a(part[i * nch + c].x - m);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     const double l2 = (double)m + log2(s);
     const double d = lse_c[n] * 1.4426950408889634 - l2;
-    audit_missed[i] = (float)fmax(0.0, -expm1(d * 0.6931471805599453));
+    if (lane == 0) audit_missed[i] = (float)fmax(0.0, -expm1(d * 0.6931471805599453));
 }
 
 __global__ void __launch_bounds__(256) k_sum_lse(const double *__restrict__ v, int64_t n, double *__restrict__ part)
@@ -1203,7 +1276,7 @@ int prop_launch_lloyd(const float *pts, int K, float *cent, SortBuffers &sb, int
                       int *cstart, int lloyd_iters, cudaStream_t st)
 {
     for (int it = 0; it <= lloyd_iters; it++) {
-        k_assign<<<(K + 255) / 256, 256, 0, st>>>(pts, K, cent, sb.keys_in, sb.idx_in);
+        k_assign<<<(K + 2 * kAssign - 1) / (2 * kAssign), kAssign, 0, st>>>(pts, K, cent, sb.keys_in, sb.idx_in);
         size_t bytes = sb.temp_bytes;
         if (cub::DeviceRadixSort::SortPairs(sb.temp, bytes, sb.keys_in, skey, sb.idx_in, order, K, 0, 11, st) !=
             cudaSuccess)
@@ -1349,9 +1422,9 @@ void prop_cand_pass2(const double *X, const double *lse_c, const float *rec32, c
                      const long long *fbase, int n_items, float *part, const int *kperm, double *dS, cudaStream_t st)
 {
     if (n_items > 0)
-        k_cand_pass2<<<(unsigned)n_items, 64, 0, st>>>(X, lse_c, rec32, order, cstart, pstart, plist, item_start,
+        k_cand_pass2<<<dim3((unsigned)n_items, kMemberSlices), 64, 0, st>>>(X, lse_c, rec32, order, cstart, pstart, plist, item_start,
                                                         fbase, part);
-    k_cand_reduce<<<kG, 128, 0, st>>>(part, rec32, order, cstart, item_start, fbase, kperm, dS);
+    k_cand_reduce<<<dim3(kG, 4), 128, 0, st>>>(part, rec32, order, cstart, item_start, fbase, kperm, dS);
 }
 
 void prop_labels(const double *Xe, const double *lse_e, const int *rows, int64_t rstride, int64_t ne,
@@ -1359,7 +1432,7 @@ void prop_labels(const double *Xe, const double *lse_e, const int *rows, int64_t
                  int64_t nb, int64_t S)
 {
     if (ne > 0)
-        k_labels<<<(unsigned)((ne * 32 + 255) / 256), 256, 0, st>>>(Xe, lse_e, rows, rstride, ne, rec32, order,
+        k_labels<<<dim3((unsigned)((ne * 32 + 255) / 256), kLabelSlices), 256, 0, st>>>(Xe, lse_e, rows, rstride, ne, rec32, order,
                                                                      cstart, UB, nb, S, Q);
 }
 
@@ -1373,7 +1446,7 @@ void prop_audit(const double *X, const int *erows, int64_t ne, const int *exact,
     float2 *part = reinterpret_cast<float2 *>(scratch);
     k_audit_part<<<dim3((unsigned)((ne + kAP - 1) / kAP), (unsigned)nch), 256, 0, st>>>(X, erows, ne, exact, rec32,
                                                                                           K, part);
-    k_audit_final<<<(unsigned)((ne + 255) / 256), 256, 0, st>>>(part, nch, erows, ne, exact, lse_c, audit_missed);
+    k_audit_final<<<(unsigned)((ne + 7) / 8), 256, 0, st>>>(part, nch, erows, ne, exact, lse_c, audit_missed);
 }
 
 void prop_lse_combine(double *lse_c, const double *lse_e, const int *erows, int64_t ne, cudaStream_t st)
