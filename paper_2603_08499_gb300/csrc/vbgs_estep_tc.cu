@@ -1143,9 +1143,12 @@ __global__ void __launch_bounds__(kPlanThreads) k_p1_plan(int64_t N, int ntiles,
 
 // ---------------------------------------------------------------------------
 // Pass 2 on the tensor cores: the fused statistics contraction of Eq. 3.
-// grid = (component tiles, N splits), 160 threads.  A CTA keeps its tile's
-// coefficients (the pass-1 tile, A operand) in shared memory and walks the
-// 64-point chunks of its split that the pass-1 bound does not rule out:
+// 160 threads, two CTAs per SM for the length of the launch.  Work items are
+// runs of one component tile's list of 64-point chunks that the pass-1 bound
+// does not rule out; a CTA walks its items as one stream of chunks, the tile's
+// coefficients (the pass-1 tile, A operand) in shared memory, so that barriers
+// and TMEM are set up once and the next item's first chunk is already in
+// flight while the last one's sums are taken.  Per chunk:
 //   MMA1  D1[128 comps x 64 pts]  = C . phi'^T      (3 hi/lo products, K = 32)
 //   epilogue (thread = component row): r = 2^(D1 * scale - lse2_n) -> P hi/lo
 //   MMA2  D2[128 comps x 32 feats]  = P_hi phi'_hi + P_hi phi'_lo + P_lo phi'_hi
@@ -1163,6 +1166,13 @@ __global__ void __launch_bounds__(kPlanThreads) k_p1_plan(int64_t N, int ntiles,
 //   B2 [32 feats x 64 pts ]: LBO 128, SBO 1024      (4 KB each for hi, lo)
 //   P  [128 comps x 64 pts]: LBO 128, SBO 1024      (16 KB each for hi, lo)
 // TMEM: D1 double buffered at columns 0 / 64, D2 double buffered at 128 / 160.
+// Bound by latency: 9 warps an SM issue in a third of the cycles, the tensor
+// cores are busy in a tenth; registers (168) and shared memory (113 KB) allow
+// no third CTA.  One CTA per item, fetching what each chunk needs where it is
+// used and taking the means through FP64, took 44.5 us a launch over the eight
+// scenes of the batched workload and 37.9 us on the 36,000-point room with
+// K = 50,000; the stream 38.6 and 32.8, frames and origins over the lanes 37.8
+// and 31.9.  Two epilogue warpgroups a CTA at 96 registers: 48.6 and 41.5.
 // ---------------------------------------------------------------------------
 constexpr int kChunk2 = 64;
 constexpr int kB1Bytes = kChunk2 * kFeat * 2;       // 4 KB
@@ -1271,16 +1281,32 @@ __global__ void __launch_bounds__(kThreadsTC, 2) k_pass2_tc(const float *__restr
     extern __shared__ unsigned char smem_raw[];
     Smem2 &S = *reinterpret_cast<Smem2 *>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // this CTA's work item: list entries [ibeg, iend) of tile j (never empty);
     // CTAs beyond the item count leave before any TMEM or barrier
-    const int item = blockIdx.x;
-    if (item >= *nitems) return;
-    const int j = item_tile[item];
+    const int n_items = *nitems;
+    if ((int)blockIdx.x >= n_items) return;
     const int64_t nchunks = (N + kChunk2 - 1) / kChunk2;
-    const int ibeg = item_lo[item], iend = item_hi[item];
-    // list entry i -> chunk index
-    auto chunk_at = [&](int i) -> int64_t { return counts ? (int64_t)list[(size_t)j * nchunks + i] : (int64_t)i; };
-    const int64_t cbeg = ibeg, cend = iend;   // iterate over list positions
+    // list entry i of tile j -> chunk index
+    auto chunk_at = [&](int j, int i) -> int { return counts ? list[(size_t)j * nchunks + i] : i; };
+    // This CTA's chunks, one stream: the list entries [lo, hi) (never empty)
+    // of its work items, item blockIdx.x and every gridDim.x-th after it; the
+    // item after the current one is read ahead.
+    struct Cursor {
+        int it, j, p, e;        // item, its tile, list position and end
+        int it2, j2, p2, e2;
+    } cur = {};
+    auto read_ahead = [&]() {
+        if (cur.it2 < n_items) { cur.j2 = item_tile[cur.it2]; cur.p2 = item_lo[cur.it2]; cur.e2 = item_hi[cur.it2]; }
+    };
+    auto advance = [&]() -> bool {   // true: a new item (it >= n_items: the end)
+        if (++cur.p < cur.e) return false;
+        cur.it = cur.it2; cur.j = cur.j2; cur.p = cur.p2; cur.e = cur.e2;
+        cur.it2 += (int)gridDim.x;
+        read_ahead();
+        return true;
+    };
+    cur.it2 = (int)blockIdx.x;
+    read_ahead();
+    advance();
 
     if (tid == 0) {
         mbar_init(&S.bar_a, 1);
@@ -1302,36 +1328,38 @@ __global__ void __launch_bounds__(kThreadsTC, 2) k_pass2_tc(const float *__restr
     __syncthreads();
     fence_after();
     const uint32_t tmem = S.tmem_base;
-    const float *h = hdr + (size_t)j * 32;
-    const float scale = h[18];
-
-    // the list holds only chunks to evaluate: positions advance one by one
-    auto next_chunk = [&](int64_t c) { return c; };
 
     if (warp < 4) {
         // ---------------- builders + responsibilities ----------------
-        const float *hf = h;   // tile frame (header), read where used (uniform, cached)
         const int m = tid;                          // component row of the epilogue
         bool ok = true;
         // The next chunk's inputs, loaded one chunk ahead of their use: this
-        // thread's point (FP32 hi/lo) and, for threads 0..63, its lse2.  The
-        // chunk origin (its first point, which thread 0 loads too) is read
-        // where it is used.
-        float nx[12], nl = INFINITY;
-        int64_t nc0 = 0;
-        // list entry of the chunk after the one load_next(c) is called for,
-        // read one call ahead
-        int64_t c0_ahead = cbeg < cend ? chunk_at((int)cbeg) * kChunk2 : 0;
-        auto load_next = [&](int64_t c) {
-            nc0 = c0_ahead;
-            if (c + 1 < cend) c0_ahead = chunk_at((int)(c + 1)) * kChunk2;
-            const int64_t n = nc0 + (tid & 63);
+        // thread's point (FP32 hi/lo) and, for threads 0..63, its lse2; over
+        // the lanes of each warp, the chunk's origin (its first point, 16
+        // floats) and its tile's header (32 floats), handed on by shuffles.
+        // Shared memory leaves L1 a few KB, so a load where the value is used
+        // is an L2 round trip.
+        float nx[12], nl = INFINITY, nxo = 0.f, nh = 0.f;
+        int nch = 0, nit = 0, nj = 0;   // its chunk, item and tile
+        // the cursor stands on the chunk after the one loaded last; its list
+        // entry is read when the cursor reaches it
+        int ch_ahead = chunk_at(cur.j, cur.p);
+        auto load_next = [&]() {
+            nch = ch_ahead;
+            nit = cur.it;
+            nj = cur.j;
+            advance();
+            if (cur.it < n_items) ch_ahead = chunk_at(cur.j, cur.p);
+            const int64_t n = (int64_t)nch * kChunk2 + (tid & 63);
             const float4 *xp = reinterpret_cast<const float4 *>(Xhl + (n < N ? n : N - 1) * 16);
             const float4 p0 = xp[0], p1 = xp[1], p2 = xp[2], p3 = xp[3];
             nx[0] = p0.x; nx[1] = p0.y; nx[2] = p0.z; nx[3] = p0.w; nx[4] = p1.x; nx[5] = p1.y;
             nx[6] = p2.x; nx[7] = p2.y; nx[8] = p2.z; nx[9] = p2.w; nx[10] = p3.x; nx[11] = p3.y;
             if (tid < 64) nl = n < N ? lse2f[n] : INFINITY;
+            nxo = Xhl[(size_t)nch * (kChunk2 * 16) + (lane & 15)];
+            nh = hdr[(size_t)nj * 32 + lane];
         };
+        auto bcast = [&](float v, int i) { return __shfl_sync(0xffffffffu, v, i); };
         auto build = [&](int st, int sl) {
             // threads 0..63 write B1 (point-major) and lse2, 64..127 write B2
             // (feature-major); each half arrives on its own barrier
@@ -1340,12 +1368,13 @@ __global__ void __launch_bounds__(kThreadsTC, 2) k_pass2_tc(const float *__restr
             if (tid < 64) {
                 // logits: the tile's frame, like the coefficients
 #pragma unroll
-                for (int i = 0; i < 6; i++) d[i] = ((nx[i] - hf[i]) + (nx[6 + i] - hf[6 + i])) * hf[12 + i];
+                for (int i = 0; i < 6; i++)
+                    d[i] = ((nx[i] - bcast(nh, i)) + (nx[6 + i] - bcast(nh, 6 + i))) * bcast(nh, 12 + i);
             } else {
                 // statistics: the chunk's frame, origin at its first point
-                const float *xo = Xhl + nc0 * 16;
 #pragma unroll
-                for (int i = 0; i < 6; i++) d[i] = ((nx[i] - xo[i]) + (nx[6 + i] - xo[8 + i])) * hf[12 + i];
+                for (int i = 0; i < 6; i++)
+                    d[i] = ((nx[i] - bcast(nxo, i)) + (nx[6 + i] - bcast(nxo, 8 + i))) * bcast(nh, 12 + i);
             }
             float f[kFeat];
             f[0] = 1.f;
@@ -1387,32 +1416,45 @@ __global__ void __launch_bounds__(kThreadsTC, 2) k_pass2_tc(const float *__restr
         // delta = o_c - m_k, per-axis scale s of the features:
         //   S1 += s S1' + N' delta,
         //   S2_ab += s_a s_b S2'_ab + delta_a s_b S1'_b + s_a S1'_a delta_b + N' delta_a delta_b.
-        float st[28];
-#pragma unroll
-        for (int i = 0; i < 28; i++) st[i] = 0.f;
-        float sc[6];
-#pragma unroll
-        for (int i = 0; i < 6; i++) sc[i] = 1.f / hf[12 + i];
-        const int kcomp = j * kCols + m;
+        float st[28], sc[6];
         float mh[6], ml[6];   // the component's mean as an FP32 hi/lo pair
-        {
-            const double *mrec = rec + (size_t)(kcomp < K ? kcomp : K - 1) * VBGS_REC;
+        int it = 0, j = 0;    // the chunk in the epilogue: item and tile
+        auto mean_row = [&]() {
+            const int kcomp = j * kCols + m;
+            return reinterpret_cast<const double2 *>(rec + (size_t)(kcomp < K ? kcomp : K - 1) * VBGS_REC);
+        };
+        float ch = 0.f;       // its tile's header, over the lanes
+        auto begin_item = [&]() {
 #pragma unroll
-            for (int i = 0; i < 6; i++) {
-                const double v = mrec[i];
-                mh[i] = (float)v;
-                ml[i] = (float)(v - (double)mh[i]);
+            for (int i = 0; i < 28; i++) st[i] = 0.f;
+#pragma unroll
+            for (int i = 0; i < 6; i++) sc[i] = 1.f / bcast(ch, 12 + i);
+            const double2 *mrec = mean_row();
+#pragma unroll
+            for (int i = 0; i < 3; i++) {
+                const double2 v = mrec[i];
+                d2f_pair(v.x, mh[2 * i], ml[2 * i]);
+                d2f_pair(v.y, mh[2 * i + 1], ml[2 * i + 1]);
             }
-        }
-        int64_t org0 = 0, org1 = 0;   // origin (first point) of the chunk in each stage
+        };
+        int fin = (int)blockIdx.x;   // the item to be written next
+        auto end_item = [&](int jt) {
+            const int item = fin;
+            fin += (int)gridDim.x;
+            if (jt * kCols + m >= K) return;
+            float4 *dst = reinterpret_cast<float4 *>(part + ((size_t)item * kCols + m) * 28);
+#pragma unroll
+            for (int i = 0; i < 7; i++) dst[i] = make_float4(st[4 * i], st[4 * i + 1], st[4 * i + 2], st[4 * i + 3]);
+        };
+        float org0 = 0.f, org1 = 0.f;   // origin of the chunk in each stage, over the lanes
         auto add_d2 = [&](int stage) {
             uint32_t v[32];
             tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + 128u + (uint32_t)(stage * kFeat), v);
             tmem_wait_ld();
-            const float *xo = Xhl + (stage ? org1 : org0) * 16;
+            const float xo = stage ? org1 : org0;
             float dl[6], s1[6];
 #pragma unroll
-            for (int i = 0; i < 6; i++) dl[i] = (xo[i] - mh[i]) + (xo[8 + i] - ml[i]);
+            for (int i = 0; i < 6; i++) dl[i] = (bcast(xo, i) - mh[i]) + (bcast(xo, 8 + i) - ml[i]);
             const float nn = __uint_as_float(v[0]);
             st[0] += nn;
 #pragma unroll
@@ -1432,18 +1474,22 @@ __global__ void __launch_bounds__(kThreadsTC, 2) k_pass2_tc(const float *__restr
         // responsibilities of chunk u from MMA1(u); (c) once MMA2(u-1) is done,
         // the statistics of chunk u-1 from D2 and B2 of chunk u+1 (threads
         // 64..127, its stage was MMA2(u-1)'s).  MMA2(u-1) thus runs while (b)
-        // computes, instead of the epilogue waiting for it.
-        const int64_t nc = cend - cbeg;
-        if (nc > 0) {
-            load_next(cbeg);
-            build(0, 0);
-            org0 = nc0;
-            if (nc > 1) load_next(cbeg + 1);
-        }
-        for (int64_t u = 0; u < nc && ok; u++) {
-            const int s = (int)(u & 1);
-            const int64_t cn = cbeg + u + 1;
-            if (cn < cend && tid < 64) build(s ^ 1, (int)((u + 1) % 3));
+        // computes, instead of the epilogue waiting for it.  An item's sums
+        // are written when its last chunk's statistics are in, one chunk into
+        // the next item.
+        load_next();
+        build(0, 0);
+        org0 = nxo;
+        it = nit; j = nj; ch = nh;
+        bool fresh = true, more = cur.it < n_items;
+        int pj = 0;   // tile of chunk u - 1
+        if (more) load_next();
+        int u = 0;
+        for (;; u++) {
+            const int s = u & 1;
+            if (more && tid < 64) build(s ^ 1, (u + 1) % 3);
+            if (fresh) asm volatile("prefetch.global.L1 [%0];" ::"l"(mean_row()));   // read in begin_item
+            const float scale = bcast(ch, 18);
             ok = __all_sync(0xffffffffu, mbar_wait(&S.bar_d1full[s], (uint32_t)((u >> 1) & 1), flags));
             if (!ok) break;
             fence_after();
@@ -1484,42 +1530,47 @@ __global__ void __launch_bounds__(kThreadsTC, 2) k_pass2_tc(const float *__restr
                 if (!ok) break;
                 fence_after();
                 add_d2(s ^ 1);
+                if (fresh) end_item(pj);
             }
-            if (cn < cend) {
-                if (tid >= 64) build(s ^ 1, (int)((u + 1) % 3));
-                if (s) org0 = nc0; else org1 = nc0;
-                if (cn + 1 < cend) load_next(cn + 1);
-            }
+            if (fresh) begin_item();
+            if (!more) break;
+            if (tid >= 64) build(s ^ 1, (u + 1) % 3);
+            if (s) org0 = nxo; else org1 = nxo;
+            pj = j;
+            fresh = nit != it;
+            it = nit; j = nj; ch = nh;
+            more = cur.it < n_items;
+            if (more) load_next();
         }
-        if (ok && nc >= 1) {
-            const int sl = (int)((nc - 1) & 1);
-            ok = __all_sync(0xffffffffu, mbar_wait(&S.bar_stfree[sl], (uint32_t)(((nc - 1) >> 1) & 1), flags));
+        if (ok) {
+            ok = __all_sync(0xffffffffu, mbar_wait(&S.bar_stfree[u & 1], (uint32_t)((u >> 1) & 1), flags));
             if (ok) {
                 fence_after();
-                add_d2(sl);
+                add_d2(u & 1);
+                end_item(j);
             }
         }
-        const int k = j * kCols + m;
-        if (k < K) {
-            float4 *dst = reinterpret_cast<float4 *>(part + ((size_t)item * kCols + m) * 28);
+        // a wait that gave up leaves zeros, not what the buffer held before
+        // (pass 1 uses it too: its log-sums are no counts)
+        if (!ok) {
 #pragma unroll
-            for (int i = 0; i < 7; i++) dst[i] = make_float4(st[4 * i], st[4 * i + 1], st[4 * i + 2], st[4 * i + 3]);
+            for (int i = 0; i < 28; i++) st[i] = 0.f;
+            while (fin < n_items) end_item(item_tile[fin]);
         }
     } else if (warp == 4 && lane == 0) {
         // ---------------- copy + MMA issuer ----------------
         constexpr uint32_t id1 = idesc_mn<BF16>(128, kChunk2);
         constexpr uint32_t id2 = idesc_mn<BF16>(128, kFeat);
         bool ok = true;
-        bool a_loaded = false;
-        int n_proc = 0;
+        int n_a = 0, n_proc = 0;   // tile copies issued, chunks whose MMA2 was issued
         bool any_mma = false;
-        int64_t c = next_chunk(cbeg);
-        if (c < cend) {
+        auto load_a = [&]() {
             mbar_expect_tx(&S.bar_a, kTileBytes);
-            bulk_g2s(S.A, tiles + (size_t)j * kTileBytes, kTileBytes, &S.bar_a);
-            a_loaded = true;
-            ok = mbar_wait(&S.bar_a, 0u, flags);
-        }
+            bulk_g2s(S.A, tiles + (size_t)cur.j * kTileBytes, kTileBytes, &S.bar_a);
+            n_a++;
+        };
+        load_a();
+        ok = mbar_wait(&S.bar_a, 0u, flags);
         auto mma1 = [&](int uu) {
             const int s = uu & 1;
             const uint32_t d = tmem + (uint32_t)(s * kChunk2);
@@ -1538,18 +1589,24 @@ __global__ void __launch_bounds__(kThreadsTC, 2) k_pass2_tc(const float *__restr
             mma_commit(&S.bar_d1full[s]);
         };
         // MMA1 of the first chunk
-        if (ok && c < cend) {
+        if (ok) {
             ok = mbar_wait(&S.bar_b1full[0], 0u, flags);
             if (ok) { fence_after(); mma1(0); any_mma = true; }
         }
-        int u = 0;
-        while (ok && c < cend) {
+        for (int u = 0; ok; u++) {
             const int s = u & 1;
-            const int64_t cn = next_chunk(c + 1);
-            if (cn < cend) {
+            const bool fresh = advance(), more = cur.it < n_items;
+            if (more) {
                 const int s1 = (u + 1) & 1;
+                if (fresh) {   // the next item's tile, once MMA1(u) has read this one's
+                    ok = mbar_wait(&S.bar_d1full[s], (uint32_t)((u >> 1) & 1), flags);
+                    if (!ok) break;
+                    fence_after();
+                    load_a();
+                }
                 ok = mbar_wait(&S.bar_b1full[s1], (uint32_t)(((u + 1) >> 1) & 1), flags) &&
-                     (u + 1 < 2 || mbar_wait(&S.bar_d1free[s1], (uint32_t)((((u + 1) >> 1) - 1) & 1), flags));
+                     (u + 1 < 2 || mbar_wait(&S.bar_d1free[s1], (uint32_t)((((u + 1) >> 1) - 1) & 1), flags)) &&
+                     (!fresh || mbar_wait(&S.bar_a, (uint32_t)((n_a - 1) & 1), flags));
                 if (!ok) break;
                 fence_after();
                 mma1(u + 1);
@@ -1572,11 +1629,10 @@ __global__ void __launch_bounds__(kThreadsTC, 2) k_pass2_tc(const float *__restr
             }
             mma_commit(&S.bar_stfree[s]);
             n_proc = u + 1;
-            c = cn;
-            u++;
+            if (!more) break;
         }
-        // Drain: last phases of the barriers the copy and the commits arrive on.
-        if (a_loaded) mbar_wait(&S.bar_a, 0u, flags, true);
+        // Drain: last phases of the barriers the copies and the commits arrive on.
+        mbar_wait(&S.bar_a, (uint32_t)((n_a - 1) & 1), flags, true);
         for (int s = 0; s < 2; s++) {
             const int last = ((n_proc - 1 - s) >= 0) ? s + ((n_proc - 1 - s) / 2) * 2 : -1;
             if (last >= 0) mbar_wait(&S.bar_stfree[s], (uint32_t)((last >> 1) & 1), flags, true);
@@ -1773,13 +1829,16 @@ int launch_pass2_tc(const float *Xhl, const float *lse2f, int64_t N, int K, bool
     const size_t smem = sizeof(Smem2) + 128;
     if (tc_set_attributes()) return -1;
     float *fpart = reinterpret_cast<float *>(part);   // item partials: FP32 register sums
+    // two CTAs resident per SM; items have nearly the same length, so every
+    // grid-th one is as good a share as the scheduler's
+    const int grid = std::min(tcap, 2 * num_sms);
     pf->begin(VBGS_PROF_PASS2, st);
     if (bf16)
-        launch_pdl(k_pass2_tc<true>, tcap, kThreadsTC, smem, st, Xhl, lse2f, N, K, tiles, hdr, ntiles, tmax ? counts : nullptr,
+        launch_pdl(k_pass2_tc<true>, grid, kThreadsTC, smem, st, Xhl, lse2f, N, K, tiles, hdr, ntiles, tmax ? counts : nullptr,
                                                          list, item_tile, item_lo, item_hi, nitems, rec, fpart, flags,
                                                          pairs, knobs);
     else
-        launch_pdl(k_pass2_tc<false>, tcap, kThreadsTC, smem, st, Xhl, lse2f, N, K, tiles, hdr, ntiles, tmax ? counts : nullptr,
+        launch_pdl(k_pass2_tc<false>, grid, kThreadsTC, smem, st, Xhl, lse2f, N, K, tiles, hdr, ntiles, tmax ? counts : nullptr,
                                                           list, item_tile, item_lo, item_hi, nitems, rec, fpart, flags,
                                                          pairs, knobs);
     pf->end(st);

@@ -30,7 +30,7 @@ __device__ double dg_digamma(double x)
     // shift = sum 1/(x + i) accumulated as one fraction num/den; one division
     // gives both shift and 1/x
     double num = 0.0, den = 1.0;
-    while (x < 10.0) { num = fma(num, x, den); den *= x; x += 1.0; }
+    for (int i = 0; i < 10 && x < 10.0; i++) { num = fma(num, x, den); den *= x; x += 1.0; }   // ends for any x
     const double r = 1.0 / (den * x);
     const double shift = num * x * r, ix = den * r;
     const double t = ix * ix;

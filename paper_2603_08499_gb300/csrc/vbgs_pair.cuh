@@ -89,4 +89,27 @@ __device__ __forceinline__ double f2d_exact(float f)
     return __longlong_as_double((long long)(sgn | ((unsigned long long)(ex + 896u) << 52) |
                                             ((unsigned long long)(b & 0x7fffffu) << 29)));
 }
+
+// FP64 -> the pair h = RN32(v), l = RN32(v - h) without an FP64 instruction
+// (each holds a warp's sub-partition for 64 cycles): the significand's top 24
+// bits rounded to nearest even, and the signed remainder of at most 2^28
+// units.  Zeros give (v, +0); values whose parts leave FP32's normal range
+// take the conversions.
+__device__ __forceinline__ void d2f_pair(double v, float &h, float &l)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const int ex = (int)((b >> 52) & 0x7ff);
+    if (ex < 949 || ex > 1149) {
+        if ((b << 1) == 0ull) { h = __uint_as_float((unsigned)(b >> 32)); l = 0.f; return; }
+        h = (float)v;
+        l = (float)(v - (double)h);
+        return;
+    }
+    const bool neg = (long long)b < 0;
+    const unsigned top = (unsigned)((b >> 29) & 0x7fffffu) | 0x800000u, rem = (unsigned)b & 0x1fffffffu;
+    const unsigned up = rem > 0x10000000u || (rem == 0x10000000u && (top & 1u)) ? 1u : 0u;
+    const int hi = (int)(top + up), lo = (int)rem - (int)(up << 29);
+    h = (float)(neg ? -hi : hi) * __uint_as_float((unsigned)(ex - 1046 + 127) << 23);
+    l = (float)(neg ? -lo : lo) * __uint_as_float((unsigned)(ex - 1075 + 127) << 23);
+}
 } // namespace vbgs
