@@ -26,9 +26,9 @@
 // Points and components come in Morton order (unless the caller keeps its
 // own), which keeps the boxes small.
 // Measured (GB300; pass 1 and pass 2, us a launch), dense -> sparse:
-//   FP64, 10,000 points, K = 1,000 (mixture):  1,226 + 2,105 -> 85 + 124
-//   FP64, 8,294 points, K = 50,000 (room):    44,100 + 8,650 -> 87 + 107
-//   FP32, 36,000 points, K = 50,000 (room):    3,472 +   982 -> 116 + 193
+//   FP64, 10,000 points, K = 1,000 (mixture):  1,226 + 2,105 -> 84 + 100
+//   FP64, 8,294 points, K = 50,000 (room):    44,100 + 8,650 -> 64 + 101
+//   FP32, 36,000 points, K = 50,000 (room):    3,472 +   982 -> 116 + 190
 // and once per frame the seeds of pass 1: 33, 76 and 117.  Bound: the FP64 pipe
 // (about 54 instructions per 32 listed pairs in pass 1, 1.7 + 1 a pair in pass
 // 2) on the mixture; latency of the record and box loads on the room.
@@ -1118,7 +1118,7 @@ __global__ void __launch_bounds__(kOneWarps * 32, 8) k_sp_pass2_one(SpView V, P2
     pdl_wait();
     constexpr bool kF64 = sizeof(T) == 8;
     constexpr int W = kOneWarps, kList2 = 64;
-    __shared__ double sacc[W * 28], ssum[28];
+    __shared__ double sacc[W * 28], ssum[2][28];
     __shared__ T srec[28];
     __shared__ float srec32[28];
     __shared__ T sx[W][32 * 7], sw[W][32 * (kF64 ? 1 : 7)];
@@ -1129,7 +1129,12 @@ __global__ void __launch_bounds__(kOneWarps * 32, 8) k_sp_pass2_one(SpView V, P2
     const int todo = A.heavy ? *A.nheavy : V.K;
     int ia, ib;
     feature_cols(lane, ia, ib);
-    for (int e = blockIdx.x / nblk; e < todo; e += ncl) {
+    // A block goes on to the cluster's next component as soon as its own sums
+    // are out; it waits for the others only before it writes the sums after
+    // those (two buffers), the first block's warp 0 before it adds them.
+    int buf = 0;
+    bool pending = false;
+    for (int e = blockIdx.x / nblk; e < todo; e += ncl, buf ^= 1) {
         const int p = A.heavy ? A.heavy[e] : e;
         if (threadIdx.x < 28) {
             srec32[threadIdx.x] = V.rec32[(size_t)p * VBGS_REC + threadIdx.x];
@@ -1262,20 +1267,24 @@ __global__ void __launch_bounds__(kOneWarps * 32, 8) k_sp_pass2_one(SpView V, P2
         if (A.pairs && lane == 0 && npair) atomicAdd(A.pairs, (unsigned long long)npair);
         if (lane < 28) sacc[w * 28 + lane] = total;
         __syncthreads();
+        if (pending) cluster.barrier_wait();
         if (threadIdx.x < 28) {
             double t = sacc[threadIdx.x];
             for (int i = 1; i < W; i++) t += sacc[i * 28 + threadIdx.x];
-            ssum[threadIdx.x] = t;
+            ssum[buf][threadIdx.x] = t;
         }
-        cluster.sync();
-        if (rank == 0 && w == 0) {
+        cluster.barrier_arrive();
+        pending = rank != 0 || w != 0;
+        if (!pending) {
+            cluster.barrier_wait();
             double t = 0.0;
             if (lane < 28)
-                for (int i = 0; i < nblk; i++) t += cluster.map_shared_rank(ssum, i)[lane];
+                for (int i = 0; i < nblk; i++) t += cluster.map_shared_rank(ssum[buf], i)[lane];
             write_row(V, A, p, t, true, srec32, lane);
         }
-        cluster.sync();   // the sums are read before the next component's
     }
+    if (pending) cluster.barrier_wait();
+    cluster.sync();   // the last sums are read before their blocks leave
 }
 
 inline size_t even(size_t v) { return (v + 3) & ~size_t(3); }
@@ -1357,12 +1366,15 @@ int launch_estep_sparse(const EstepBuffers &B, int precision, bool want_stats, i
         }
     }
     // FP64: four warps a block, and a cluster per point group until the grid
-    // holds eight blocks an SM.  FP32: one block per group, with warps enough
+    // holds five blocks an SM: fewer leave the FP64 pipe idle in the tail, more
+    // cut the lists into partly filled batches (clusters of 1 / 2 / 4 / 8, us a
+    // launch: 313 groups 96 / 94 / 84 / 102, 386 groups 173 / 147 / 154 / 183,
+    // 254 groups of the room 107 / 76 / 64 / 86).  FP32: one block per group, with warps enough
     // for about four a sub-partition (more would cut the grid into two waves).
     // Component groups are cut into units until every warp has a few.
     int W = 4, cl = 1;
     if (f64)
-        while (cl < kCluster && V.G * cl < 8 * num_sms && 8 * cl <= 4 * V.Kg) cl *= 2;
+        while (cl < kCluster && V.G * cl < 5 * num_sms && 8 * cl <= 4 * V.Kg) cl *= 2;
     else
         while (W < kP1Warps && (int64_t)V.G * W < 4 * (int64_t)num_sms * 4 && 2 * W <= 4 * V.Kg) W *= 2;
     int nsub = 1;
@@ -1409,10 +1421,21 @@ int launch_estep_sparse(const EstepBuffers &B, int precision, bool want_stats, i
         launches++;
     }
     pf->begin(VBGS_PROF_PASS2, st);
-    // a round of blocks (eight resident an SM), whose clusters take turns;
-    // FP32: a warp per split is all a component can use
+    // A round of blocks (eight resident an SM), whose clusters take turns.
+    // FP64: clusters of eight while there are few components, smaller ones as
+    // soon as they would need over four rounds, since a block evaluates its
+    // lists in batches of 32 pairs and small shares leave the batches part
+    // filled (clusters of 1 / 2 / 4 / 8, us a launch: K = 64 45 / 28 / 21 / 20,
+    // K = 1,000 129 / 103 / 98 / 124, K = 1,777 196 / 169 / 199 / 279); the
+    // heavy components of a wide map take four (2 / 4 / 8: 36 / 30 / 37).
+    // FP32: a warp per split is all a component can use, and the heavy ones of
+    // a wide map are enough to fill the chip (1 / 2 / 4 / 8: 132 / 145 / 195 /
+    // 299).
     cl = kCluster;
-    while (!f64 && cl > 1 && cl / 2 * kOneWarps >= p2_splits) cl /= 2;
+    if (f64)
+        while (wide ? cl > 4 : cl > 1 && (int64_t)V.K * cl > 32 * num_sms) cl /= 2;
+    else
+        while (cl > 1 && (wide || cl / 2 * kOneWarps >= p2_splits)) cl /= 2;
     const int clusters = std::max(1, std::min(8 * num_sms / cl, V.K));
     if (f64) launch_pdl_cluster(k_sp_pass2_one<double>, clusters * cl, kOneWarps * 32, cl, 0, st, V, a2);
     else     launch_pdl_cluster(k_sp_pass2_one<float>, clusters * cl, kOneWarps * 32, cl, 0, st, V, a2);
