@@ -800,11 +800,14 @@ __global__ void __launch_bounds__(128) k_p1_ub(const float *__restrict__ boxes, 
     const int k = j * kCols + t;
     const int nv = min(kCols, K - j * kCols);
     {
-        const float *r = rec32 + (size_t)(k < K ? k : 0) * VBGS_REC;
+        // the floats used of the 128-byte row (0-5, 27-30), four loads in
+        // flight (282 point tiles, K = 50,000: 16.6 -> 15.0 us)
+        const float4 *r4 = reinterpret_cast<const float4 *>(rec32 + (size_t)(k < K ? k : 0) * VBGS_REC);
+        const float4 ra = r4[0], rb = r4[1], rc = r4[6], rd = r4[7];
+        const float r[10] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rc.w, rd.x, rd.y, rd.z};
         float v[16];
 #pragma unroll
-        for (int i = 0; i < 6; i++) sc[t][i] = r[i];
-        sc[t][6] = r[27]; sc[t][7] = r[28]; sc[t][8] = r[29]; sc[t][9] = r[30];
+        for (int i = 0; i < 10; i++) sc[t][i] = r[i];
         // group summary over the valid components of this warp's 32
         const bool valid = t < nv;
 #pragma unroll
@@ -812,9 +815,9 @@ __global__ void __launch_bounds__(128) k_p1_ub(const float *__restrict__ boxes, 
             v[i] = valid ? r[i] : INFINITY;
             v[6 + i] = valid ? r[i] : -INFINITY;
         }
-        v[12] = valid ? r[27] : -INFINITY;
+        v[12] = valid ? r[6] : -INFINITY;
 #pragma unroll
-        for (int i = 0; i < 3; i++) v[13 + i] = valid ? r[28 + i] : INFINITY;
+        for (int i = 0; i < 3; i++) v[13 + i] = valid ? r[7 + i] : INFINITY;
 #pragma unroll
         for (int i = 0; i < 16; i++) {
             const bool mx = i >= 6 && i <= 12;
