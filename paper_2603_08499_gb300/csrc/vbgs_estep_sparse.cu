@@ -29,6 +29,7 @@
 //   FP64, 10,000 points, K = 1,000 (mixture):  1,226 + 2,105 -> 84 + 100
 //   FP64, 8,294 points, K = 50,000 (room):    44,100 + 8,650 -> 64 + 101
 //   FP32, 36,000 points, K = 50,000 (room):    3,472 +   982 -> 116 + 190
+//   FP32, 6,500 points, K = 1,500 (mixture):      52 +   110 -> 67 + 49
 // and once per frame the seeds of pass 1: 33, 76 and 117.  Bound: the FP64 pipe
 // (about 54 instructions per 32 listed pairs in pass 1, 1.7 + 1 a pair in pass
 // 2) on the mixture; latency of the record and box loads on the room.
@@ -1436,14 +1437,17 @@ int launch_estep_sparse(const EstepBuffers &B, int precision, bool want_stats, i
     // filled (clusters of 1 / 2 / 4 / 8, us a launch: K = 64 45 / 28 / 21 / 20,
     // K = 1,000 129 / 103 / 98 / 124, K = 1,777 196 / 169 / 199 / 279); the
     // heavy components of a wide map take four (2 / 4 / 8: 36 / 30 / 37).
-    // FP32: a warp per split is all a component can use, and the heavy ones of
-    // a wide map are enough to fill the chip (1 / 2 / 4 / 8: 132 / 145 / 195 /
-    // 299).
+    // FP32: a warp per split is all a component can use, with a few pairs each,
+    // so clusters of two from 300 components on (1 / 2 / 4 / 8: K = 300 57 / 36 /
+    // 39 / 41, K = 700 51 / 45 / 47 / 57, K = 1,500 55 / 49 / 67 / 101, K = 2,200
+    // 56 / 58 / 79 / 138); the heavy components of a wide map are enough to fill
+    // the chip alone (132 / 145 / 195 / 299).
     cl = kCluster;
-    if (f64)
-        while (wide ? cl > 4 : cl > 1 && (int64_t)V.K * cl > 32 * num_sms) cl /= 2;
-    else
-        while (cl > 1 && (wide || cl / 2 * kOneWarps >= p2_splits)) cl /= 2;
+    auto crowded = [&]() {
+        if (wide) return f64 ? cl > 4 : true;
+        return (int64_t)V.K * cl > (f64 || cl <= 2 ? 32 : 4) * num_sms || (!f64 && cl / 2 * kOneWarps >= p2_splits);
+    };
+    while (cl > 1 && crowded()) cl /= 2;
     const int clusters = std::max(1, std::min(8 * num_sms / cl, V.K));
     if (f64) launch_pdl_cluster(k_sp_pass2_one<double>, clusters * cl, kOneWarps * 32, cl, 0, st, V, a2);
     else     launch_pdl_cluster(k_sp_pass2_one<float>, clusters * cl, kOneWarps * 32, cl, 0, st, V, a2);
